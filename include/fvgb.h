@@ -64,7 +64,9 @@ typedef enum {
 /* Arithmetic of the face computations.  The state in memory is always IEEE
  * binary64 and the residual sum and RK update keep binary64 accuracy. */
 typedef enum {
-  FV_PREC_FP64 = 0,      /* every operation in IEEE binary64 */
+  FV_PREC_FP64 = 0,      /* IEEE binary64; the Roe flux of a face in 64-bit
+                            fixed point with the face's own scales where the
+                            face fits them (error below binary64's) */
   FV_PREC_DF64 = 1,      /* face arithmetic in double-float (pairs of binary32,
                             ~48-bit significand) on the FP32 pipe */
   FV_PREC_FP32FLUX = 2   /* limiter / reconstruction / Roe flux in binary32;

@@ -16,7 +16,8 @@ STAGE_VARIANTS = [form + fast + visc + bc for form in ("fp64", "df64", "fp32") f
                   for visc in ("", "_visc") for bc in ("", "_bc")]
 SOURCES = ["fv_stage_%s.cu" % v for v in STAGE_VARIANTS] + [
     "fv_api.cu", "fv_noalloc.cu", "fv_probe.cu", "fv_adjoint.cu", "fv_visc.cu", "fv_monitor.cu"]
-HEADERS = ["fv_arith.cuh", "fv_face.cuh", "fv_stage.cuh", "fv_viscface.cuh", "fv_internal.h", "fv_adjoint.cuh"]
+HEADERS = ["fv_arith.cuh", "fv_face.cuh", "fv_stage.cuh", "fv_viscface.cuh", "fv_internal.h", "fv_adjoint.cuh",
+           "fv_fixed.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
 

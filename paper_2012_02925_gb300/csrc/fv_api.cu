@@ -32,6 +32,7 @@ struct fv_ctx {
   int ntiles = 0;
   int* d_tile_counter = nullptr;    // dynamic tile scheduling of the stage kernel
   FvLaunch launch{};
+  FxConsts fx{};                    // constants of the binary64 form's fixed-point Roe flux
   FvConnDev* d_conns = nullptr;
   long long conn_items = 0;
   FvXchTile* d_xtiles = nullptr;    // exchange kernel work units of d_conns
@@ -728,6 +729,7 @@ FvStageArgs base_args(fv_ctx* h) {
   a.fp.limiter = h->cfg.limiter;
   a.fp.fix_all = h->cfg.fix_all;
   a.fp.flux = h->cfg.flux;
+  a.fp.fx = h->fx;
   if (h->launch.visc && h->cfg.precision == FV_PREC_FP32FLUX) {
     // binary32: viscous terms fused into the stage kernel
     a.geo = h->geo_t;
@@ -1197,6 +1199,7 @@ int fv_create_blocks(const fv_block_desc* blocks, int nblocks, const fv_connecti
   h->nblocks = nblocks;
   h->nconn = nconn;
   h->conns.assign(conns, conns + nconn);
+  h->fx = fx_consts(cfg->gamma, cfg->harten);
   cudaError_t e = cudaGetDevice(&h->device);
   if (e != cudaSuccess) return fail(nullptr, FV_ERR_CUDA, std::string("cudaGetDevice: ") + cudaGetErrorString(e));
   cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->device);

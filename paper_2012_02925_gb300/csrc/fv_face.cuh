@@ -25,6 +25,7 @@ struct FaceC {
   int limiter, fix_all, has_fix;
   int upwind_only;  // kappa == -1: the (1+kappa) terms of Eq. (flux) vanish
   int unit_slope;   // eps (1 - kappa) / 2 == 1: the upwind slope enters with weight one
+  FxConsts fx;
   // the scheme switches as the face code reads them
   __device__ __forceinline__ int k_flux() const { return flux; }
   __device__ __forceinline__ int k_lim() const { return limiter; }
@@ -80,6 +81,7 @@ __device__ __forceinline__ FaceC<T> make_face_consts(const FvFaceParams& p) {
   c.has_fix = p.harten > 0.0;
   c.upwind_only = (p.kappa == -1.0);
   c.unit_slope = (p.eps * 0.5 * (1.0 - p.kappa) == 1.0);
+  c.fx = p.fx;
   return c;
 }
 
@@ -287,7 +289,14 @@ __device__ __forceinline__ void steger_warming_part(const CC& C, const T V[5], T
 template <class T, class CC>
 __device__ __forceinline__ void face_riemann(const CC& C, const T VL[5], const T VR[5], T nx, T ny, T nz, T A,
                                              T out[5]) {
-  if (C.k_flux() == 0) { roe_flux(C, VL, VR, nx, ny, nz, A, out); return; }
+  if (C.k_flux() == 0) {
+    // binary64: on the integer units where the face fits (fv_fixed.cuh)
+    if constexpr (std::is_same<T, double>::value) {
+      if (C.fx.on && fx_roe_flux(C.fx, VL, VR, nx, ny, nz, A, C.k_fixall(), out)) return;
+    }
+    roe_flux(C, VL, VR, nx, ny, nz, A, out);
+    return;
+  }
   T Fp[5], Fm[5];
   if (C.k_flux() == 1) {
     vanleer_part(C, VL, nx, ny, nz, +1, Fp);

@@ -2,6 +2,7 @@
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
+#include "fv_fixed.cuh"
 
 #define FV_GHOST 2
 
@@ -71,6 +72,7 @@ struct FvViscParams {
 struct FvFaceParams {
   double gamma, eps, kappa, harten, va_delta2;
   int limiter, fix_all, flux;
+  FxConsts fx;                  // the binary64 form's fixed-point Roe flux
 };
 
 enum { FV_MODE_RK = 0, FV_MODE_RESIDUAL = 1 };
