@@ -107,6 +107,8 @@ __device__ __forceinline__ void prim_from_cons(const CC& C, const T q[5], T V[5]
 template <class T>
 __device__ __forceinline__ T vanleer_half(T a, T b) {
   using S = Sc<T>;
+  // binary64: on the integer units
+  if constexpr (std::is_same<T, double>::value) return fx_vanleer_half(a, b);
   const T p = a * b, s = a + b;
   const T h = S::div(p, s);
   return S::sel(S::pos(p) && S::above(S::abs(s), 1e-30f), h, S::c(0.0));

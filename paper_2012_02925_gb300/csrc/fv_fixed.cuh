@@ -3,9 +3,8 @@
 //
 // GB300's FP64 unit issues 1.6 lanes per SM and clock, so one binary64
 // operation occupies 80 of an SM's 128-lane issue slots; a signed 64 x 64 ->
-// high 64 bit product costs 23 (three IMAD.HI at 4.5, one IMAD, the carries)
-// and a 64-bit sum 3 (measured on the part; an unsigned wide IMAD 4.6, a
-// signed one 9).  Every quantity of the face is held with an absolute
+// high 64 bit product costs about 23 (two IMAD.HI at 4.5, a signed wide IMAD
+// at 9, the carries) and a 64-bit sum 3 (measured on the part).  Every quantity of the face is held with an absolute
 // resolution of 2^-60 .. 2^-71 of the face's scales, so that a flux carries
 // 2^-55 .. 2^-57 of its terms, where binary64 rounds each of its ~126
 // operations to 2^-53.
@@ -54,17 +53,7 @@ FX_HD void fx_split(fx64 a, int& h, int& l) {
   l = (int)a;
   h = (int)(a >> 32) + (int)((unsigned)l >> 31);
 }
-// the exact signed product of two 32-bit numbers; as low and high halves (the
-// signed wide multiply runs at half the rate of the two together)
-FX_HD fx64 fx_prod(int a, int b) {
-#ifdef __CUDA_ARCH__
-  const unsigned lo = (unsigned)a * (unsigned)b;
-  const int hi = fx_madhi(a, b, 0);
-  return (fx64)(((fxu64)(unsigned)hi << 32) | lo);
-#else
-  return (fx64)a * b;
-#endif
-}
+FX_HD fx64 fx_prod(int a, int b) { return (fx64)a * b; }
 // a b / 2^64 for |a|, |b| < 2^63 - 2^31: the product of the low halves is left
 // out and the two cross products are rounded down (error within 2.3 units;
 // zero times anything is zero)
@@ -438,6 +427,68 @@ FX_HD double fx_to_double(fx64 x, int e) {
 #else
   return ldexp((double)x, e);
 #endif
+}
+
+FX_HD double fx_double(int hi, unsigned lo) {
+#ifdef __CUDA_ARCH__
+  return __hiloint2double(hi, (int)lo);
+#else
+  const fxu64 b = ((fxu64)(unsigned)hi << 32) | lo;
+  double d;
+  __builtin_memcpy(&d, &b, 8);
+  return d;
+#endif
+}
+
+// Half the van Leer limited slope of differences a, b: a b/(a + b) when they
+// have the same sign, else 0, within 0.65 units in the last place; 0 when
+// both are below 2^-100 (rounding noise of a quantity that is zero).  The
+// significands' product over their aligned sum, by a 32-bit reciprocal (the
+// hardware's approximation, one Newton step) and one correction.  About 140
+// issue slots where the six binary64 operations (product, sum, reciprocal of
+// three, product) hold the FP64 unit for 480.  128^3 RK step: 5.83 -> 4.28 ms (autotuned),
+// 64-block batch: 49.2 -> 39.4 ms.
+FX_HD double fx_vanleer_half(double a, double b) {
+  const int ha = fx_hi(a), hb = fx_hi(b);
+  const unsigned la = fx_lo(a), lb = fx_lo(b);
+  const int ea = (ha >> 20) & 0x7ff, eb = (hb >> 20) & 0x7ff;
+  const unsigned ah = ((((unsigned)ha & 0xfffffu) | 0x100000u) << 10) | (la >> 22), al = la << 10;
+  const unsigned bh = ((((unsigned)hb & 0xfffffu) | 0x100000u) << 10) | (lb >> 22), bl = lb << 10;
+  const fxu64 A = ((fxu64)ah << 32) | al, B = ((fxu64)bh << 32) | bl;   // [2^62, 2^63): a = A 2^(ea - 1085)
+  const int em = ea > eb ? ea : eb, en = ea > eb ? eb : ea;
+  const int d = em - en;
+  const fxu64 big = ea > eb ? A : B, small = ea > eb ? B : A;
+  const fxu64 S0 = big + (d < 64 ? small >> (d & 63) : 0);              // [2^62, 2^64)
+  const int n = (int)(~(unsigned)(S0 >> 32) >> 31);
+  const fxu64 S = S0 << n;                                              // s' = S / 2^64 in [1/2, 1)
+  const unsigned sh = (unsigned)(S >> 32), sl = (unsigned)S;
+  // r = 2^30 / s': 1/f of f = 2 s' to 22 bits, then a Newton step
+  const float f = fx_asfloat((int)(0x3f800000u | ((sh >> 8) & 0x7fffffu)));
+#ifdef __CUDA_ARCH__
+  const float g = __fmaf_rn(fx_rcpf(f), 4194302.0f, 8388608.0f);        // 2^23 + 2^22 / f (r0 below 2^31)
+#else
+  const float g = fmaf(fx_rcpf(f), 4194302.0f, 8388608.0f);
+#endif
+  const unsigned r0 = ((unsigned)fx_asint(g) & 0x7fffffu) << 9;         // 2^31 / f = 2^30 / s'
+  const int e1 = (int)(0x40000000u - fx_umulhi(sh, r0));
+  const unsigned r = r0 + (unsigned)fx_madhi((int)r0, e1 * 4, 0);
+  const fx64 e2 = (fx64)(0x4000000000000000ull - ((fxu64)sh * r + fx_umulhi(sl, r)));   // |e2| < 2^34
+  const fxu64 P = (fxu64)fx_umul((fx64)A, (fx64)B);                     // [2^60, 2^62)
+  const fxu64 H0 = ((fxu64)(unsigned)(P >> 32) * r + fx_umulhi((unsigned)P, r)) << 2;   // P / s', below 2^63
+  const fxu64 H = H0 + (fxu64)((fx64)fx_madhi((int)(H0 >> 32), (int)(e2 >> 3), 0) << 5);
+  // round to 53 bits: significand m (implicit bit 52) times 2^(e - 1075)
+#ifdef __CUDA_ARCH__
+  const int z = __clz((int)(unsigned)(H >> 32));
+#else
+  const int z = __builtin_clz((unsigned)(H >> 32));
+#endif
+  const fxu64 N = H << z;
+  const fxu64 m = (N >> 11) + ((N >> 10) & 1);
+  const int e = en + 1 - z + n;                                         // ea + eb - em + 1 - z + n
+  const fxu64 bits = m + ((fxu64)(unsigned)(e - 1) << 52);
+  const bool zero = (ha ^ hb) < 0 || em < 923 || en < 64;
+  const int hh = (int)(bits >> 32) | (ha & (int)0x80000000);
+  return fx_double(zero ? 0 : (em == 2047 ? 0x7ff80000 : hh), zero ? 0u : (unsigned)bits);
 }
 
 // Roe flux times the area A of the states VL, VR along the unit normal n in

@@ -1,5 +1,6 @@
-"""The binary64 form's fixed-point Roe flux (csrc/fv_fixed.cuh), compiled for
-the host, against the oracle's binary64 one.
+"""The binary64 form's fixed-point Roe flux and integer slope quotient
+(csrc/fv_fixed.cuh), compiled for the host: the flux against the oracle's
+binary64 one, the slope against exact rationals.
 
 Tolerance, derived before the first run: the oracle's ~130 binary64 operations
 and its inputs' rounding leave at most ~16 units of 2^-53 of the flux's scale
@@ -24,6 +25,7 @@ extern "C" int fixed_roe(double gamma, double harten, int fix_all, const double*
   const FxConsts c = fx_consts(gamma, harten);
   return c.on ? (int)fx_roe_flux(c, L, R, n[0], n[1], n[2], A, fix_all != 0, out) : -1;
 }
+extern "C" double half_slope(double a, double b) { return fx_vanleer_half(a, b); }
 '''
 
 
@@ -44,6 +46,9 @@ def fixed(tmp_path_factory):
         rc = L.fixed_roe(gamma, harten, fix_all, *(x.ctypes.data_as(dp) for x in a), A, out.ctypes.data_as(dp))
         return rc, out
 
+    L.half_slope.argtypes = [ctypes.c_double] * 2
+    L.half_slope.restype = ctypes.c_double
+    call.slope = L.half_slope
     return call
 
 
@@ -114,3 +119,25 @@ def test_refuses_what_does_not_fit(fixed):
         assert fixed(base, base, [1.0, 0.0, 0.0], A)[0] == 0
     assert fixed(base, base, [1.0, 0.0, 0.0], 1.0, gamma=1.1)[0] == -1
     assert fixed(base, base, [1.0, 0.0, 0.0], 1.0, harten=0.01)[0] == -1
+
+
+def test_half_slope(fixed):
+    """a b / (a + b) of differences with the same sign, else 0, within one
+    unit in the last place of the exact quotient (rationals)."""
+    from fractions import Fraction
+    f = fixed.slope
+    rng = np.random.default_rng(5)
+    edge = [1.0, 2.0, 1.0 - 2.0 ** -53, 2.0 - 2.0 ** -52, 1.5, 1.0 + 2.0 ** -52]
+    pairs = [(a * 2.0 ** i, b) for a in edge for b in edge for i in (0, 1, 10, 53, 62, 63, 64, 70)]
+    pairs += [(x, y) for x, y in zip(rng.uniform(0.5, 2, 3000) * 2.0 ** rng.integers(-40, 40, 3000),
+                                     rng.uniform(0.5, 2, 3000))]
+    for a, b in pairs:
+        for x, y in ((a, b), (b, a), (-a, -b)):
+            want = Fraction(x) * Fraction(y) / (Fraction(x) + Fraction(y))
+            got = f(x, y)
+            assert abs(Fraction(got) - want) <= Fraction(float(np.spacing(abs(float(want))))), (x, y, got)
+        assert f(a, -b) == 0.0 and f(-a, b) == 0.0
+    assert f(0.0, 1.0) == 0.0 and f(1.0, 0.0) == 0.0 and f(0.0, 0.0) == 0.0
+    assert f(4e-31, 4e-31) == 0.0 and f(1e-300, 1.0) <= 1e-300
+    for bad in (np.nan, np.inf):
+        assert np.isnan(f(bad, 1.0)) and np.isnan(f(1.0, bad))
