@@ -152,25 +152,46 @@ FV_HD df64 df_dot(const df64 (&a)[N], const df64 (&b)[N]) {
   return quick_two_sum(s, err);
 }
 
-__device__ __forceinline__ float fv_rcp(float x) { return __frcp_rn(x); }
+// binary32 reciprocal within about half a unit in the last place: the
+// hardware's approximation and one Newton step (the IEEE reciprocal is a
+// multi-instruction sequence with special-case branches; the callers' operands
+// are normal numbers, or the result is discarded)
+__device__ __forceinline__ float fv_rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return FFMA(r, FFMA(-x, r, 1.0f), r);
+}
 
-// a / b: correctly rounded binary32 reciprocal of b.hi, quotient estimate and
-// one correction step in double-float (relative error ~2^-47)
+// a / b: quotient estimate q1 of the high parts, its remainder a - b q1 by
+// fused multiply-adds (the high parts' is exact up to its last bit), and the
+// correction q2.  Error as the IEEE reciprocal with a double-float remainder
+// gives (rms 3.2e-15, at most 3.2e-14 of the quotient), at 11 instructions
+// instead of 37: 128^3 double-float RK step 3.00 -> 2.73 ms, the 151x49x27
+// O-grid's 0.635 -> 0.536 ms
 FV_HD df64 operator/(df64 a, df64 b) {
-  float r = fv_rcp(b.hi);
-  float q1 = FMUL(a.hi, r);
-  df64 rem = a - b * q1;
-  float q2 = FMUL(rem.hi, r);
+  const float r = fv_rcp(b.hi);
+  const float q1 = FMUL(a.hi, r);
+  const float e = FFMA(-q1, b.hi, a.hi);
+  const float q2 = FMUL(FFMA(-q1, b.lo, FADD(e, a.lo)), r);
   return quick_two_sum(q1, q2);
 }
-FV_HD df64 df_rcp(df64 b) { return mk(1.0f, 0.0f) / b; }
+FV_HD df64 df_rcp(df64 b) {
+  const float r = fv_rcp(b.hi);
+  return quick_two_sum(r, FMUL(FFMA(-r, b.lo, FFMA(-r, b.hi, 1.0f)), r));
+}
 
+// square root: the hardware's approximate reciprocal square root, one coupled
+// Newton step for s ~ sqrt(a.hi) and h ~ 1/(2 s), then the remainder a - s^2
+// (error as from the IEEE binary32 root: rms 1.4e-15, at most 1.4e-14)
 FV_HD df64 df_sqrt(df64 a) {
   if (!(a.hi > 0.0f)) return mk(a.hi == 0.0f ? 0.0f : __int_as_float(0x7fc00000), 0.0f);
-  float s = __fsqrt_rn(a.hi);
-  df64 e = a - two_prod(s, s);
-  float corr = FMUL(e.hi, FMUL(0.5f, __fdividef(1.0f, s)));
-  return quick_two_sum(s, corr);
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a.hi));
+  const float s0 = FMUL(a.hi, y), h0 = FMUL(0.5f, y);
+  const float d = FFMA(-s0, h0, 0.5f);
+  const float s = FFMA(s0, d, s0), h = FFMA(h0, d, h0);
+  const float e = FADD(FFMA(-s, s, a.hi), a.lo);
+  return quick_two_sum(s, FMUL(e, h));
 }
 FV_HD df64 df_abs(df64 a) { return a.hi < 0.0f ? -a : a; }
 FV_HD bool operator<(df64 a, df64 b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
