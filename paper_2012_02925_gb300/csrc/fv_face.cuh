@@ -14,6 +14,7 @@
 template <class T>
 struct FaceC {
   T gm1;          // gamma - 1
+  T eps;          // MUSCL eps
   T g_gm1;        // gamma / (gamma - 1)
   T half, one;
   T e4km, e4kp;   // eps/4 (1 - kappa), eps/4 (1 + kappa)
@@ -60,6 +61,7 @@ __device__ __forceinline__ FaceC<T> make_face_consts(const FvFaceParams& p) {
   using S = Sc<T>;
   FaceC<T> c;
   c.gm1 = S::c(p.gamma - 1.0);
+  c.eps = S::c(p.eps);
   c.g_gm1 = S::c(p.gamma / (p.gamma - 1.0));
   c.half = S::c(0.5);
   c.one = S::c(1.0);
@@ -127,6 +129,29 @@ __device__ __forceinline__ T limited(const CC& C, T a, T b) {
   const T a2 = a * a;
   const T num = b * (a2 + a * b);
   return num * S::rcp(a2 + b * b + C.va_d2);
+}
+
+// The half-slope h of a cell with forward and backward differences a, b: for
+// the two symmetric limiters, Psi(a/b) b = Psi(b/a) a, both terms of Eq.
+// (flux) are the same limited difference and kappa drops out,
+// V + eps/2 Psi(a/b) b on the cell's upper face and V - the same on its lower.
+// The unlimited scheme's two terms differ: its faces take the backward
+// difference from here and the other two from the ring (unlimited_states).
+template <class CC>
+__device__ __forceinline__ double cell_slope(const CC& C, double a, double b) {
+  if (std::is_same<CC, FaceCFast<double>>::value) return vanleer_half(a, b);
+  if (C.k_lim() == 1) return C.eps * vanleer_half(a, b);
+  if (C.k_lim() == 0) return b;
+  const double p = a * b, s = a + b;
+  return fx_div((0.5 * C.eps) * p * s, s * s - 2.0 * p + C.va_d2);
+}
+
+// Eq. (flux) without a limiter, from the backward difference dm of V_i
+template <class T, class CC>
+__device__ __forceinline__ void unlimited_states(const CC& C, T dm, T v0, T vp1, T vp2, T& L, T& R) {
+  const T d0 = vp1 - v0, dp = vp2 - vp1;
+  L = v0 + (C.e4km * dm + C.e4kp * d0);
+  R = vp1 - (C.e4kp * d0 + C.e4km * dp);
 }
 
 // Eq. (flux) for one component from V_{i-1}, V_i, V_{i+1}, V_{i+2}

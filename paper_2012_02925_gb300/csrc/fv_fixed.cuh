@@ -440,6 +440,61 @@ FX_HD double fx_double(int hi, unsigned lo) {
 #endif
 }
 
+// 2^30 / s' for s' = (2^32 sh + sl) / 2^64 in [1/2, 1): 32 bits (the hardware's
+// approximation to 22 bits, one Newton step), and e2 = 2^62 (1 - s' r / 2^30),
+// |e2| < 2^34
+FX_HD unsigned fx_rcp32(unsigned sh, unsigned sl, fx64& e2) {
+  const float f = fx_asfloat((int)(0x3f800000u | ((sh >> 8) & 0x7fffffu)));   // 2 s'
+#ifdef __CUDA_ARCH__
+  const float g = __fmaf_rn(fx_rcpf(f), 4194302.0f, 8388608.0f);        // 2^23 + 2^22 / f (r0 below 2^31)
+#else
+  const float g = fmaf(fx_rcpf(f), 4194302.0f, 8388608.0f);
+#endif
+  const unsigned r0 = ((unsigned)fx_asint(g) & 0x7fffffu) << 9;         // 2^31 / f = 2^30 / s'
+  const int e1 = (int)(0x40000000u - fx_umulhi(sh, r0));
+  const unsigned r = r0 + (unsigned)fx_madhi((int)r0, e1 * 4, 0);
+  e2 = (fx64)(0x4000000000000000ull - ((fxu64)sh * r + fx_umulhi(sl, r)));
+  return r;
+}
+// P / s' from the reciprocal above, P in [2^60, 2^63): the product and its correction
+FX_HD fxu64 fx_quot(fxu64 P, unsigned r, fx64 e2) {
+  const fxu64 H0 = ((fxu64)(unsigned)(P >> 32) * r + fx_umulhi((unsigned)P, r)) << 2;
+  return H0 + (fxu64)((fx64)fx_madhi((int)(H0 >> 32), (int)(e2 >> 3), 0) << 5);
+}
+// H 2^(e - 1086), H >= 2^32, rounded to binary64's 53 bits: its pattern
+// without a sign (the exponent in the normal range)
+FX_HD fxu64 fx_round(fxu64 H, int e) {
+#ifdef __CUDA_ARCH__
+  const int z = __clz((int)(unsigned)(H >> 32));
+#else
+  const int z = __builtin_clz((unsigned)(H >> 32));
+#endif
+  const fxu64 N = H << z;
+  return (N >> 11) + ((N >> 10) & 1) + ((fxu64)(unsigned)(e - 1 - z) << 52);
+}
+
+// n / d for a finite d > 0, within 0.65 units in the last place; a quotient
+// below the normal range is 0, above it infinite, of a non-finite n NaN
+FX_HD double fx_div(double n, double d) {
+  const int hn = fx_hi(n), hd = fx_hi(d);
+  const unsigned ln = fx_lo(n), ld = fx_lo(d);
+  const int en = (hn >> 20) & 0x7ff, ed = (hd >> 20) & 0x7ff;
+  const unsigned dh = ((((unsigned)hd & 0xfffffu) | 0x100000u) << 11) | (ld >> 21), dl = ld << 11;   // [2^63, 2^64)
+  const fxu64 P = ((fxu64)(((((unsigned)hn & 0xfffffu) | 0x100000u) << 9) | (ln >> 23)) << 32) | (ln << 9);   // [2^61, 2^62)
+  fx64 e2;
+  const unsigned r = fx_rcp32(dh, dl, e2);
+  const fxu64 H = fx_quot(P, r, e2);                                    // [2^61, 2^63)
+  // n = P 2^(en - 1084), d = s' 2^64 2^(ed - 1086): H 2^(en - ed - 62)
+  const int e = en - ed + 1024;
+  const fxu64 b = fx_round(H, e);
+  const int sg = hn & (int)0x80000000;
+  const bool nan = en == 2047 || ed == 2047 || hd <= 0;
+  const bool zero = en == 0 || e < 4;
+  const bool inf = (unsigned)(b >> 52) >= 2047u;
+  const int hi = nan ? 0x7ff80000 : (zero ? sg : (inf ? sg | 0x7ff00000 : sg | (int)(b >> 32)));
+  return fx_double(hi, nan || zero || inf ? 0u : (unsigned)b);
+}
+
 // Half the van Leer limited slope of differences a, b: a b/(a + b) when they
 // have the same sign, else 0, within 0.65 units in the last place; 0 when
 // both are below 2^-100 (rounding noise of a quantity that is zero).  The
@@ -461,31 +516,11 @@ FX_HD double fx_vanleer_half(double a, double b) {
   const fxu64 S0 = big + (d < 64 ? small >> (d & 63) : 0);              // [2^62, 2^64)
   const int n = (int)(~(unsigned)(S0 >> 32) >> 31);
   const fxu64 S = S0 << n;                                              // s' = S / 2^64 in [1/2, 1)
-  const unsigned sh = (unsigned)(S >> 32), sl = (unsigned)S;
-  // r = 2^30 / s': 1/f of f = 2 s' to 22 bits, then a Newton step
-  const float f = fx_asfloat((int)(0x3f800000u | ((sh >> 8) & 0x7fffffu)));
-#ifdef __CUDA_ARCH__
-  const float g = __fmaf_rn(fx_rcpf(f), 4194302.0f, 8388608.0f);        // 2^23 + 2^22 / f (r0 below 2^31)
-#else
-  const float g = fmaf(fx_rcpf(f), 4194302.0f, 8388608.0f);
-#endif
-  const unsigned r0 = ((unsigned)fx_asint(g) & 0x7fffffu) << 9;         // 2^31 / f = 2^30 / s'
-  const int e1 = (int)(0x40000000u - fx_umulhi(sh, r0));
-  const unsigned r = r0 + (unsigned)fx_madhi((int)r0, e1 * 4, 0);
-  const fx64 e2 = (fx64)(0x4000000000000000ull - ((fxu64)sh * r + fx_umulhi(sl, r)));   // |e2| < 2^34
-  const fxu64 P = (fxu64)fx_umul((fx64)A, (fx64)B);                     // [2^60, 2^62)
-  const fxu64 H0 = ((fxu64)(unsigned)(P >> 32) * r + fx_umulhi((unsigned)P, r)) << 2;   // P / s', below 2^63
-  const fxu64 H = H0 + (fxu64)((fx64)fx_madhi((int)(H0 >> 32), (int)(e2 >> 3), 0) << 5);
-  // round to 53 bits: significand m (implicit bit 52) times 2^(e - 1075)
-#ifdef __CUDA_ARCH__
-  const int z = __clz((int)(unsigned)(H >> 32));
-#else
-  const int z = __builtin_clz((unsigned)(H >> 32));
-#endif
-  const fxu64 N = H << z;
-  const fxu64 m = (N >> 11) + ((N >> 10) & 1);
-  const int e = en + 1 - z + n;                                         // ea + eb - em + 1 - z + n
-  const fxu64 bits = m + ((fxu64)(unsigned)(e - 1) << 52);
+  fx64 e2;
+  const unsigned r = fx_rcp32((unsigned)(S >> 32), (unsigned)S, e2);
+  const fxu64 H = fx_quot((fxu64)fx_umul((fx64)A, (fx64)B), r, e2);     // product in [2^60, 2^62)
+  // h = H 2^(n + ea + eb - em - 1085)
+  const fxu64 bits = fx_round(H, en + 1 + n);
   const bool zero = (ha ^ hb) < 0 || em < 923 || en < 64;
   const int hh = (int)(bits >> 32) | (ha & (int)0x80000000);
   return fx_double(zero ? 0 : (em == 2047 ? 0x7ff80000 : hh), zero ? 0u : (unsigned)bits);

@@ -101,24 +101,28 @@ struct StageSmem {
 // makes h symmetric in a and b, so the two faces share one limiter
 // evaluation, done once per cell and direction in a slope pass before the
 // faces (about 0.56 of the per-face stencil's limiter work with the tile
-// halo).  Built for the binary64 form, which the FP64 unit bounds (128^3
-// block: 0.625 -> 0.716 Gcell/s); the double-float and binary32 forms are
-// bound by issue and latency at their occupancy, and the slope planes, the
-// third barrier per plane and the lost resident CTA made them slower
-// (2.75 -> 2.62 and 9.84 -> 8.26 Gcell/s), so they keep the per-face stencil.
-template <class T, bool FAST, bool VISC>
+// halo).  The same holds for every kappa and eps with either limiter
+// (cell_slope), so every binary64 kernel takes its slopes so (128^3 block,
+// default scheme: 0.625 -> 0.716 Gcell/s; van
+// Albada with kappa = 1/3 and the van Leer splitting, 97x61x53 residual: 1.01
+// -> 0.61 ms; the Roe flux with van Albada 0.83 -> 0.43 ms).
+// The double-float and binary32 forms are bound by issue and latency at their
+// occupancy, and the slope planes, the third barrier per plane and the lost
+// resident CTA made them slower (2.75 -> 2.62 and 9.84 -> 8.26 Gcell/s), so
+// they keep the per-face stencil.
+template <class T>
 __host__ __device__ constexpr bool stage_share() {
-  return FAST && std::is_same<T, double>::value;
+  return std::is_same<T, double>::value;
 }
 // planes in the 3-D ring: with shared slopes a pass reads planes k .. k+2
 // only, unless a slip-wall zeta face on a block's upper side reads k - 1
-template <class T, bool FAST, bool VISC, bool BC>
+template <class T, bool BC>
 __host__ __device__ constexpr int stage_slots() {
-  return stage_share<T, FAST, VISC>() && !BC ? 3 : 4;
+  return stage_share<T>() && !BC ? 3 : 4;
 }
 template <class T, int TX, int TY, bool FAST, bool VISC, bool BC>
 using StageSmemOf = StageSmem<T, TX, TY, (VISC && std::is_same<T, float>::value) ? 6 : 5,
-                              stage_share<T, FAST, VISC>(), stage_slots<T, FAST, VISC, BC>()>;
+                              stage_share<T>(), stage_slots<T, BC>()>;
 
 // resident CTAs per SM the register allocation must allow (shared memory
 // permits this many for the compiled shapes)
@@ -145,12 +149,12 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   using AT = typename Acc<T>::type;
   using MT = typename MetricStore<T>::type;
   constexpr int NV = FUSED_VISC ? 6 : 5;
-  constexpr bool SHARE = stage_share<T, FAST, VISC>();
+  constexpr bool SHARE = stage_share<T>();
   using SM = StageSmemOf<T, TX, TY, FAST, VISC, BC>;
   constexpr int W = SM::W, PL = SM::PL;
   constexpr int NXI = SM::NXI, NETA = SM::NETA, NZETA = SM::NZETA;
   constexpr int NHX = SM::NHX, NHY = SM::NHY;
-  constexpr int NSLOT = DIM3 ? stage_slots<T, FAST, VISC, BC>() : 1;
+  constexpr int NSLOT = DIM3 ? stage_slots<T, BC>() : 1;
   constexpr int NFACE = NXI + NETA + (DIM3 ? NZETA : 0);
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -315,10 +319,15 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         normal_face_flux(C, Vb, nx, ny, nz, A, out);
       } else if constexpr (SHARE) {
         T VL[5], VR[5];
+        if (FAST || C.k_lim() != 0) {
 #pragma unroll
-        for (int n = 0; n < 5; ++n) {
-          VL[n] = s1[n * PL] + hL[n * hs];
-          VR[n] = s2[n * PL] - hR[n * hs];
+          for (int n = 0; n < 5; ++n) {
+            VL[n] = s1[n * PL] + hL[n * hs];
+            VR[n] = s2[n * PL] - hR[n * hs];
+          }
+        } else {
+#pragma unroll
+          for (int n = 0; n < 5; ++n) unlimited_states(C, hL[n * hs], s1[n * PL], s2[n * PL], s3[n * PL], VL[n], VR[n]);
         }
         face_riemann(C, VL, VR, nx, ny, nz, A, out);
       } else {
@@ -389,7 +398,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         }
       }
     };
-    // SHARE: the half-slopes h = vanleer_half(forward, backward difference)
+    // SHARE: the half-slopes h = cell_slope(forward, backward difference)
     // of the cells the faces read - in xi and eta those of plane kp (cells
     // x = -1 .. TX, rows y = -1 .. TY, inside the ghosted block), in zeta
     // that of plane kz (from planes kz-1 .. kz+1, into the slot of kz's
@@ -432,7 +441,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
 #pragma unroll
         for (int n = 0; n < 5; ++n) {
           const T v0 = c0[n * PL];
-          hd[n * hs] = vanleer_half(cp[n * PL] - v0, v0 - cm[n * PL]);
+          if constexpr (SHARE) hd[n * hs] = cell_slope(C, cp[n * PL] - v0, v0 - cm[n * PL]);
         }
       }
     };

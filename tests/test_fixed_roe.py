@@ -26,6 +26,7 @@ extern "C" int fixed_roe(double gamma, double harten, int fix_all, const double*
   return c.on ? (int)fx_roe_flux(c, L, R, n[0], n[1], n[2], A, fix_all != 0, out) : -1;
 }
 extern "C" double half_slope(double a, double b) { return fx_vanleer_half(a, b); }
+extern "C" double quotient(double n, double d) { return fx_div(n, d); }
 '''
 
 
@@ -49,6 +50,9 @@ def fixed(tmp_path_factory):
     L.half_slope.argtypes = [ctypes.c_double] * 2
     L.half_slope.restype = ctypes.c_double
     call.slope = L.half_slope
+    L.quotient.argtypes = [ctypes.c_double] * 2
+    L.quotient.restype = ctypes.c_double
+    call.quotient = L.quotient
     return call
 
 
@@ -141,3 +145,19 @@ def test_half_slope(fixed):
     assert f(4e-31, 4e-31) == 0.0 and f(1e-300, 1.0) <= 1e-300
     for bad in (np.nan, np.inf):
         assert np.isnan(f(bad, 1.0)) and np.isnan(f(1.0, bad))
+
+
+def test_quotient(fixed):
+    """n / d, d > 0, within one unit in the last place over binary64's normal
+    range; zero, overflow and what is not finite."""
+    f = fixed.quotient
+    rng = np.random.default_rng(6)
+    edge = [1.0, 2.0, 1.0 - 2.0 ** -53, 2.0 - 2.0 ** -52, 1.5, 1.0 + 2.0 ** -52]
+    pairs = [(a * 2.0 ** i, b * 2.0 ** j) for a in edge for b in edge for i in (-500, 0, 500) for j in (-500, 0, 500)]
+    pairs += list(zip(rng.uniform(-2, 2, 4000), rng.uniform(1e-3, 2, 4000)))
+    for n, d in pairs:
+        assert abs(f(n, d) - n / d) <= np.spacing(abs(n / d)), (n, d)
+    assert f(0.0, 3.0) == 0.0 and f(1e300, 1e-300) == np.inf and f(-1e300, 1e-300) == -np.inf
+    assert f(1e-300, 1e300) == 0.0 and f(1.7e308, 1.0) == 1.7e308
+    for n, d in ((np.nan, 1.0), (1.0, np.nan), (np.inf, 1.0), (1.0, np.inf), (1.0, 0.0), (1.0, -1.0)):
+        assert np.isnan(f(n, d))
