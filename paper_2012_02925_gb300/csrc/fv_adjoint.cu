@@ -3,12 +3,21 @@
 // with X the ghost exchange.  For a cotangent lam of Q^(m):
 //   mu_c   = -alpha_m dt / Omega_c * lam_c              (cotangent of R_c)
 //   Fbar_f = mu_L(f) - mu_R(f)                          (R_L holds +F_f, R_R holds -F_f)
-//   qbar   = sum over faces of (dF_f/dq)^T Fbar_f        (face_vjp, 4-cell stencil)
+//   per face: cotangents of its two states from Fbar_f    (roe_vjp)
+//   per cell: slopes and primitive recovery transposed    (adj_cell_kernel)
 //   ghost cotangents are added into their donor cells (transpose of X),
 //   fixed ghosts are constants.
-// Deterministic: per-face contributions go to a scratch array and every cell
-// gathers its (up to 12) contributions in a fixed order; connections are
-// transposed one launch at a time in table order.
+// Deterministic: the faces' cotangents go to a scratch array and every cell
+// gathers its own in a fixed order; connections are transposed one launch at
+// a time in table order.
+//
+// 96^3 VJP stage (van Albada), double-float sweeps 1.80 -> 0.98 ms, binary64
+// 4.58 -> 4.13 ms against one kernel per face that recovered its four cells'
+// primitives, evaluated the limiter's derivatives (20 of them), and reversed
+// all of it into 20 conserved cotangents (12,700 instructions a face, 160
+// bytes written): a face now does its Roe part and writes 10 cotangents
+// component by component; limiter derivatives and the recovery's transpose
+// are taken per cell.
 #include "fv_adjoint.cuh"
 #include "fv_internal.h"
 
@@ -18,128 +27,204 @@ __device__ __forceinline__ long long ghost_index(const FvBlockDev& B, int i, int
   return (long long)(k + FV_GHOST) * B.kstride + (long long)(j + FV_GHOST) * B.jstride + (i + FV_GHOST);
 }
 
-// faces of direction `dir` in block B: index f over (n_dir + 1) x (other two
-// extents); the face's VJP in arithmetic T, inputs and outputs binary64
-// NT threads per CTA; PARK: values dead across the Roe part parked in shared
-// memory (ADJ_PARK per thread); LOCK: the CTA's warps pass barriers at fixed
-// points of every face VJP (every thread runs the same number of faces, the
-// last ones repeating the final face without storing it)
-template <class T, int NT, int MINB, bool PARK, bool LOCK>
-__global__ void __launch_bounds__(NT, MINB) adj_face_kernel(const FvBlockDev B, int dir, const double* __restrict__ qin,
+// storage of an arithmetic type's values (8 bytes either way)
+template <class T> struct AdjMem;
+template <> struct AdjMem<double> {
+  using type = double;
+  static __device__ __forceinline__ double ld(const double* p) { return __ldg(p); }
+  static __device__ __forceinline__ void st(double* p, double v) { *p = v; }
+};
+template <> struct AdjMem<df64> {
+  using type = float2;
+  static __device__ __forceinline__ df64 ld(const float2* p) {
+    const float2 v = __ldg(p);
+    return mk(v.x, v.y);
+  }
+  static __device__ __forceinline__ void st(float2* p, df64 v) { *p = make_float2(v.hi, v.lo); }
+};
+
+// Primitive variables of every ghosted cell of the block, once: a face and a
+// cell sweep each read a cell's primitives up to twelve times.  (Corner
+// ghosts hold no data; nothing reads theirs.)
+template <class T>
+__global__ void adj_prim_kernel(const FvBlockDev B, const double* __restrict__ qin, const AdjParams PP,
+                                typename AdjMem<T>::type* __restrict__ prim) {
+  using S = Sc<T>;
+  using M = AdjMem<T>;
+  const AdjC<T> P = adj_consts<T>(PP);
+  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < B.plane;
+       x += (long long)gridDim.x * blockDim.x) {
+    T q[5];
+#pragma unroll
+    for (int n = 0; n < 5; ++n) q[n] = S::from_d(__ldg(qin + B.qoff + x + n * B.plane));
+    const PrimFwd<T> s = prim_fwd(P, q);
+    typename M::type* o = prim + B.qoff + x;
+    M::st(o, s.r);
+    M::st(o + B.plane, s.u);
+    M::st(o + 2 * B.plane, s.v);
+    M::st(o + 3 * B.plane, s.w);
+    M::st(o + 4 * B.plane, s.p);
+  }
+}
+
+// The faces of direction `dir` of block B, (n_dir + 1) x (the other two
+// extents): MUSCL states, then the cotangents of VL and VR from the Roe
+// sweep, stored component by component (out[c * nf + f], c = 0..4 for VL,
+// 5..9 for VR).  What the MUSCL reconstruction and the primitive recovery
+// pass on is taken per cell (adj_cell_kernel), where it is needed once per
+// cell and direction instead of four times per face.
+template <class T, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) adj_face_kernel(const FvBlockDev B, int dir,
+                                                       const typename AdjMem<T>::type* __restrict__ prim,
                                                        const double* __restrict__ lam_out,
                                                        const double* __restrict__ invvol, double alpha_dt,
-                                                       const double* __restrict__ metric, long long mstride,
-                                                       const AdjParams PP, double* __restrict__ contrib) {
+                                                       const double* __restrict__ metric, const AdjParams PP,
+                                                       typename AdjMem<T>::type* __restrict__ out) {
   using S = Sc<T>;
+  using M = AdjMem<T>;
   const AdjC<T> P = adj_consts<T>(PP);
   const int ei = B.ni + (dir == 0), ej = B.nj + (dir == 1), ek = B.nk + (dir == 2);
   const long long nf = (long long)ei * ej * ek;
   const long long ncell_b = (long long)B.ni * B.nj * B.nk;
   const double* lam = lam_out + 5 * B.cell_off;
-  const double* qb = qin + B.qoff;
-  for (long long base = blockIdx.x * (long long)NT; base < nf; base += (long long)gridDim.x * NT) {
-    const bool valid = base + threadIdx.x < nf;
-    if (!LOCK && !valid) break;
-    const long long f = valid ? base + threadIdx.x : nf - 1;
-    const int i = (int)(f % ei), j = (int)((f / ei) % ej), k = (int)(f / ((long long)ei * ej));
-    const int g = dir == 0 ? i : (dir == 1 ? j : k);            // face between cells g-1 and g
-    const int n_dir = dir == 0 ? B.ni : (dir == 1 ? B.nj : B.nk);
-    const long long stride = dir == 0 ? 1 : (dir == 1 ? B.jstride : B.kstride);
-    const long long c1 = ghost_index(B, i - (dir == 0), j - (dir == 1), k - (dir == 2));   // cell g-1
-    T q[4][5];
+  const long long f = blockIdx.x * (long long)NT + threadIdx.x;
+  if (f >= nf) return;
+  const int i = (int)(f % ei), j = (int)((f / ei) % ej), k = (int)(f / ((long long)ei * ej));
+  const int g = dir == 0 ? i : (dir == 1 ? j : k);            // face between cells g-1 and g
+  const int n_dir = dir == 0 ? B.ni : (dir == 1 ? B.nj : B.nk);
+  const long long stride = dir == 0 ? 1 : (dir == 1 ? B.jstride : B.kstride);
+  const long long c1 = ghost_index(B, i - (dir == 0), j - (dir == 1), k - (dir == 2));   // cell g-1
+  const typename M::type* v = prim + B.qoff + c1;
+  T VL[5], VR[5];
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
-#pragma unroll
-      for (int n = 0; n < 5; ++n) q[s][n] = S::from_d(qb[c1 + (s - 1) * stride + n * B.plane]);
-    // cotangent of the face flux from the two cells' residual cotangents
-    double Fd[5] = {0, 0, 0, 0, 0};
-    if (g - 1 >= 0) {
-      const int il = i - (dir == 0), jl = j - (dir == 1), kl = k - (dir == 2);
-      const long long cl = ((long long)kl * B.nj + jl) * B.ni + il;
-      const double fac = -alpha_dt * (B.cartesian ? B.cart_invvol : invvol[B.cell_off + cl]);
-#pragma unroll
-      for (int n = 0; n < 5; ++n) Fd[n] += fac * lam[n * ncell_b + cl];
-    }
-    if (g < n_dir) {
-      const long long cr = ((long long)k * B.nj + j) * B.ni + i;
-      const double fac = -alpha_dt * (B.cartesian ? B.cart_invvol : invvol[B.cell_off + cr]);
-#pragma unroll
-      for (int n = 0; n < 5; ++n) Fd[n] -= fac * lam[n * ncell_b + cr];
-    }
-    T Fb[5];
-#pragma unroll
-    for (int n = 0; n < 5; ++n) Fb[n] = S::from_d(Fd[n]);
-    T nx, ny, nz, A;
-    if (B.cartesian) {
-      nx = S::from_d(B.cart_n[dir][0]); ny = S::from_d(B.cart_n[dir][1]); nz = S::from_d(B.cart_n[dir][2]);
-      A = S::from_d(B.cart_area[dir]);
+  for (int n = 0; n < 5; ++n) {
+    const T v0 = M::ld(v - stride + n * B.plane), v1 = M::ld(v + n * B.plane);
+    const T v2 = M::ld(v + stride + n * B.plane), v3 = M::ld(v + 2 * stride + n * B.plane);
+    const T dm = v1 - v0, d0 = v2 - v1, dp = v3 - v2;
+    if (P.limiter != 0) {
+      VL[n] = v1 + P.e2 * lim_value(P, d0, dm);
+      VR[n] = v2 - P.e2 * lim_value(P, d0, dp);
     } else {
-      const long long fi = B.face_off[dir] + f;
-      nx = S::from_d(metric[4 * fi]); ny = S::from_d(metric[4 * fi + 1]);
-      nz = S::from_d(metric[4 * fi + 2]); A = S::from_d(metric[4 * fi + 3]);
+      VL[n] = v1 + S::dot2(P.e4km, dm, P.e4kp, d0);
+      VR[n] = v2 - S::dot2(P.e4kp, d0, P.e4km, dp);
     }
-    T qbar[4][5], F[5];
+  }
+  // cotangent of the face flux from the two cells' residual cotangents
+  double Fd[5] = {0, 0, 0, 0, 0};
+  if (g - 1 >= 0) {
+    const int il = i - (dir == 0), jl = j - (dir == 1), kl = k - (dir == 2);
+    const long long cl = ((long long)kl * B.nj + jl) * B.ni + il;
+    const double fac = -alpha_dt * (B.cartesian ? B.cart_invvol : invvol[B.cell_off + cl]);
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+    for (int n = 0; n < 5; ++n) Fd[n] += fac * lam[n * ncell_b + cl];
+  }
+  if (g < n_dir) {
+    const long long cr = ((long long)k * B.nj + j) * B.ni + i;
+    const double fac = -alpha_dt * (B.cartesian ? B.cart_invvol : invvol[B.cell_off + cr]);
 #pragma unroll
-      for (int n = 0; n < 5; ++n) qbar[s][n] = S::c(0.0);
-    if constexpr (PARK) {
-      extern __shared__ __align__(16) unsigned char adj_smem[];
-      T* park = reinterpret_cast<T*>(adj_smem) + threadIdx.x;
-      face_vjp<T, NT, LOCK>(P, q, nx, ny, nz, A, Fb, qbar, F, park);
-    } else {
-      face_vjp<T, 0, LOCK>(P, q, nx, ny, nz, A, Fb, qbar, F);
-    }
-    if (!valid) continue;
-    double* out = contrib + f * 20;
+    for (int n = 0; n < 5; ++n) Fd[n] -= fac * lam[n * ncell_b + cr];
+  }
+  T Fb[5];
 #pragma unroll
-    for (int s = 0; s < 4; ++s)
+  for (int n = 0; n < 5; ++n) Fb[n] = S::from_d(Fd[n]);
+  T nx, ny, nz, A;
+  if (B.cartesian) {
+    nx = S::from_d(B.cart_n[dir][0]); ny = S::from_d(B.cart_n[dir][1]); nz = S::from_d(B.cart_n[dir][2]);
+    A = S::from_d(B.cart_area[dir]);
+  } else {
+    const long long fi = B.face_off[dir] + f;
+    nx = S::from_d(metric[4 * fi]); ny = S::from_d(metric[4 * fi + 1]);
+    nz = S::from_d(metric[4 * fi + 2]); A = S::from_d(metric[4 * fi + 3]);
+  }
+  T Lb[5], Rb[5];
+  roe_vjp(P, VL, VR, nx, ny, nz, A, Fb, Lb, Rb);
 #pragma unroll
-      for (int n = 0; n < 5; ++n) out[s * 5 + n] = S::to_d(qbar[s][n]);
+  for (int n = 0; n < 5; ++n) {
+    M::st(out + n * nf + f, Lb[n]);
+    M::st(out + (5 + n) * nf + f, Rb[n]);
   }
 }
 
-// every ghosted cell: sum its face contributions, xi then eta then zeta,
-// faces in increasing order within a direction
-__global__ void adj_gather_kernel(const FvBlockDev B, const double* __restrict__ cx, const double* __restrict__ cy,
-                                  const double* __restrict__ cz, int three_d, double* __restrict__ lamg) {
+// Every ghosted cell's cotangent: per direction, the cell's own face states
+// V + h and V - h (h the limited half-slope of its forward difference a and
+// backward difference b) and its neighbours' slopes; then the primitive
+// recovery's transpose.  With Lb, Rb the cotangents of a cell's two face
+// states, alpha = dh/da (Lb - Rb) and beta = dh/db (Lb - Rb) (the unlimited
+// scheme's two slopes differ), the cell at p gets
+//   Lb + Rb - alpha(p) + beta(p) + alpha(p-1) - beta(p+1).
+// Fixed order of summation: xi, eta, zeta; deterministic.
+template <class T>
+__global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const typename AdjMem<T>::type* __restrict__ prim,
+                                                       const typename AdjMem<T>::type* __restrict__ cx,
+                                                       const typename AdjMem<T>::type* __restrict__ cy,
+                                                       const typename AdjMem<T>::type* __restrict__ cz, int three_d,
+                                                       const AdjParams PP, double* __restrict__ lamg) {
+  using S = Sc<T>;
+  using M = AdjMem<T>;
+  const AdjC<T> P = adj_consts<T>(PP);
   const int gi = B.ni + 2 * FV_GHOST, gj = B.nj + 2 * FV_GHOST, gk = B.nk + 2 * FV_GHOST;
   const long long n = (long long)gi * gj * gk;
-  double* out = lamg + B.qoff;
-  for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < n; x += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(x % gi) - FV_GHOST, j = (int)((x / gi) % gj) - FV_GHOST, k = (int)(x / ((long long)gi * gj)) - FV_GHOST;
-    const bool ii = i >= 0 && i < B.ni, jj = j >= 0 && j < B.nj, kk = k >= 0 && k < B.nk;
-    double acc[5] = {0, 0, 0, 0, 0};
-    if (jj && kk) {
-      for (int s = 3; s >= 0; --s) {              // faces g = i+2-s in increasing order
-        const int g = i + 2 - s;
-        if (g < 0 || g > B.ni) continue;
-        const double* c = cx + ((((long long)k * B.nj + j) * (B.ni + 1)) + g) * 20 + s * 5;
+  const long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (x >= n) return;
+  const int i = (int)(x % gi) - FV_GHOST, j = (int)((x / gi) % gj) - FV_GHOST, k = (int)(x / ((long long)gi * gj)) - FV_GHOST;
+  const bool ii = i >= 0 && i < B.ni, jj = j >= 0 && j < B.nj, kk = k >= 0 && k < B.nk;
+  const typename M::type* v = prim + B.qoff + x;
+  T Vb[5];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) acc[v] += c[v];
+  for (int m = 0; m < 5; ++m) Vb[m] = S::c(0.0);
+#pragma unroll 1
+  for (int dir = 0; dir < 2 + three_d; ++dir) {
+    if (!(dir == 0 ? jj && kk : (dir == 1 ? ii && kk : ii && jj))) continue;
+    const int p = dir == 0 ? i : (dir == 1 ? j : k), nd = dir == 0 ? B.ni : (dir == 1 ? B.nj : B.nk);
+    const long long st = dir == 0 ? 1 : (dir == 1 ? B.jstride : B.kstride);
+    const typename M::type* c = dir == 0 ? cx : (dir == 1 ? cy : cz);
+    // face g = p's index, and the distance of two faces along the direction
+    const long long ei = B.ni + (dir == 0), ej = B.nj + (dir == 1), ek = B.nk + (dir == 2);
+    const long long nf = ei * ej * ek, fs = dir == 0 ? 1 : (dir == 1 ? ei : ei * ej);
+    const long long f0 = ((long long)k * ej + j) * ei + i;
+    // cells p-1, p, p+1 with a face state: -1 .. nd
+#pragma unroll
+    for (int o = -1; o <= 1; ++o) {
+      const int m = p + o;
+      if (m < -1 || m > nd) continue;
+      const bool up = m + 1 <= nd, lo = m >= 0;                 // its upper and lower face exist
+#pragma unroll 1
+      for (int q = 0; q < 5; ++q) {
+        const T L = up ? M::ld(c + q * nf + f0 + (o + 1) * fs) : S::c(0.0);
+        const T R = lo ? M::ld(c + (5 + q) * nf + f0 + o * fs) : S::c(0.0);
+        const typename M::type* w = v + q * B.plane + o * st;
+        const T vm = M::ld(w - st), v0 = M::ld(w), vp = M::ld(w + st);
+        T al, be;
+        if (P.limiter != 0) {
+          T da, db;
+          lim_derivatives(P, vp - v0, v0 - vm, da, db);
+          const T d = P.e2 * (L - R);
+          al = d * da;
+          be = d * db;
+        } else {
+          al = P.e4kp * L - P.e4km * R;
+          be = P.e4km * L - P.e4kp * R;
+        }
+        const T add = o == 0 ? (L + R) - (al - be) : (o < 0 ? al : -be);
+#pragma unroll
+        for (int z = 0; z < 5; ++z) Vb[z] = z == q ? Vb[z] + add : Vb[z];
       }
     }
-    if (ii && kk) {
-      for (int s = 3; s >= 0; --s) {
-        const int g = j + 2 - s;
-        if (g < 0 || g > B.nj) continue;
-        const double* c = cy + ((((long long)k * (B.nj + 1) + g) * B.ni) + i) * 20 + s * 5;
-#pragma unroll
-        for (int v = 0; v < 5; ++v) acc[v] += c[v];
-      }
-    }
-    if (three_d && ii && jj) {
-      for (int s = 3; s >= 0; --s) {
-        const int g = k + 2 - s;
-        if (g < 0 || g > B.nk) continue;
-        const double* c = cz + ((((long long)g * B.nj + j) * B.ni) + i) * 20 + s * 5;
-#pragma unroll
-        for (int v = 0; v < 5; ++v) acc[v] += c[v];
-      }
-    }
-#pragma unroll
-    for (int v = 0; v < 5; ++v) out[x + v * B.plane] = acc[v];
   }
+  // the cell's primitives and the transpose of the recovery
+  PrimFwd<T> s;
+  s.r = M::ld(v);
+  s.u = M::ld(v + B.plane);
+  s.v = M::ld(v + 2 * B.plane);
+  s.w = M::ld(v + 3 * B.plane);
+  s.ri = S::rcp(s.r);
+  s.k = S::dot3(s.u, s.u, s.v, s.v, s.w, s.w);
+  T qb[5];
+  prim_bwd(P, s, Vb, qb);
+  double* o = lamg + B.qoff + x;
+  const bool any = (ii && jj) || (ii && kk) || (jj && kk);
+#pragma unroll
+  for (int m = 0; m < 5; ++m) o[m * B.plane] = any ? S::to_d(qb[m]) : 0.0;
 }
 
 // transpose of one connection: donor interior cell += ghost cotangent
@@ -196,49 +281,50 @@ int grid_of(long long n, int threads) {
 
 }  // namespace
 
-int fv_adjoint_faces(const FvBlockDev& B, int dir, const double* qin, const double* lam_out, const double* invvol,
-                     double alpha_dt, const double* metric, long long mstride, const FvFaceParams& fp,
-                     int double_float, double* contrib, cudaStream_t s) {
+namespace {
+AdjParams adj_params(const FvFaceParams& fp) {
   AdjParams P;
   P.gm1 = fp.gamma - 1.0;
   P.g_gm1 = fp.gamma / (fp.gamma - 1.0);
   P.e4km = fp.eps * 0.25 * (1.0 - fp.kappa);
   P.e4kp = fp.eps * 0.25 * (1.0 + fp.kappa);
+  P.e2 = fp.eps * 0.5;
   P.harten = fp.harten;
   P.va_d2 = fp.va_delta2;
   P.limiter = fp.limiter;
   P.fix_all = fp.fix_all;
-  const long long nf = (long long)(B.ni + (dir == 0)) * (B.nj + (dir == 1)) * (B.nk + (dir == 2));
-  // The double-float sweep parks its cell primitives, MUSCL states and
-  // Jacobian in shared memory across the Roe part (55 KB per CTA of 128
-  // threads), runs the MUSCL forward as a loop, is capped at 128 registers
-  // for 4 CTAs per SM (~200 bytes spill) and the warps of a CTA pass
-  // barriers at five points of each face.  96^3 VJP stage on GB300: 2.52 ms
-  // (168 registers, 430 bytes spilled, 3 CTAs) -> 2.29 (parked, 3 CTAs, no
-  // spill) -> 2.03 (parked, 4 CTAs) -> 1.97 (barriers) -> 1.80 ms (MUSCL
-  // loop); one CTA of 384 threads (168 registers, no spill) took 2.34 ms,
-  // two of 256 1.98 ms.  The binary64 sweep is bound by the FP64 unit and
-  // keeps its registers.
-  if (double_float) {
-    constexpr int NT = 128, MB = 4;
-    constexpr bool LOCK = true;
-    constexpr int smem = ADJ_PARK * sizeof(df64) * NT;
-    if (smem > 48 * 1024)
-      cudaFuncSetAttribute(adj_face_kernel<df64, NT, MB, true, LOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    adj_face_kernel<df64, NT, MB, true, LOCK><<<grid_of(nf, NT), NT, smem, s>>>(B, dir, qin, lam_out, invvol, alpha_dt,
-                                                                             metric, mstride, P, contrib);
-  } else {
-    adj_face_kernel<double, 128, 1, false, false><<<grid_of(nf, 128), 128, 0, s>>>(B, dir, qin, lam_out, invvol,
-                                                                                  alpha_dt, metric, mstride, P, contrib);
-  }
-  return cudaGetLastError() == cudaSuccess ? 0 : -1;
+  return P;
 }
 
-int fv_adjoint_gather(const FvBlockDev& B, const double* cx, const double* cy, const double* cz, int three_d,
-                      double* lamg, cudaStream_t s) {
+template <class T, int MINB>
+int adjoint_block(const FvBlockDev& B, int nd, const double* qin, const double* lam_out, const double* invvol,
+                  double alpha_dt, const double* const metric[3], const FvFaceParams& fp, void* prim_mem, void* cot_mem,
+                  double* lamg, cudaStream_t s) {
+  using MT = typename AdjMem<T>::type;
+  const AdjParams P = adj_params(fp);
+  MT* prim = static_cast<MT*>(prim_mem);
+  adj_prim_kernel<T><<<grid_of(B.plane, 256), 256, 0, s>>>(B, qin, P, prim);
+  MT* c[3] = {static_cast<MT*>(cot_mem), nullptr, nullptr};
+  for (int d = 0; d < nd; ++d) {
+    const long long nf = (long long)(B.ni + (d == 0)) * (B.nj + (d == 1)) * (B.nk + (d == 2));
+    if (d) {
+      const long long before = (long long)(B.ni + (d == 1)) * (B.nj + (d == 2)) * B.nk;
+      c[d] = c[d - 1] + 10 * before;
+    }
+    adj_face_kernel<T, 128, MINB><<<(unsigned)((nf + 127) / 128), 128, 0, s>>>(B, d, prim, lam_out, invvol, alpha_dt,
+                                                                             metric[d], P, c[d]);
+  }
   const long long n = (long long)(B.ni + 4) * (B.nj + 4) * (B.nk + 4);
-  adj_gather_kernel<<<grid_of(n, 256), 256, 0, s>>>(B, cx, cy, cz, three_d, lamg);
+  adj_cell_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(B, prim, c[0], c[1], c[2], nd == 3, P, lamg);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+}  // namespace
+
+int fv_adjoint_block(const FvBlockDev& B, int nd, const double* qin, const double* lam_out, const double* invvol,
+                     double alpha_dt, const double* const metric[3], const FvFaceParams& fp, int double_float,
+                     void* prim, void* cot, double* lamg, cudaStream_t s) {
+  return double_float ? adjoint_block<df64, 4>(B, nd, qin, lam_out, invvol, alpha_dt, metric, fp, prim, cot, lamg, s)
+                      : adjoint_block<double, 3>(B, nd, qin, lam_out, invvol, alpha_dt, metric, fp, prim, cot, lamg, s);
 }
 
 int fv_adjoint_transpose(const FvBlockDev* d_blocks, const FvConnDev& c, double* lamg, cudaStream_t s) {

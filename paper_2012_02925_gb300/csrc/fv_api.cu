@@ -52,7 +52,8 @@ struct fv_ctx {
   bool staged = false;
   double* partials = nullptr;       // per-CTA norm partials
   double* d_norm = nullptr;         // 11 doubles
-  double* adj_contrib = nullptr;    // adjoint: per-face input cotangents (20 per face)
+  double* adj_prim = nullptr;       // adjoint: primitive variables of the stage input
+  double* adj_cot = nullptr;        // adjoint: cotangents of the face states, one block at a time (10 per face)
   double* adj_lamg = nullptr;       // adjoint: ghosted cotangent of Q^(m-1)
   double* adj_qx = nullptr;         // adjoint: X(Q^(m-1)), the exchanged stage input
   int adj_df64 = 0;                 // adjoint face VJPs in double-float arithmetic (fv_set_adjoint_arith)
@@ -1388,7 +1389,7 @@ int fv_destroy(fv_handle hh) {
   cudaFree(h->d_blocks); cudaFree(h->d_tiles); cudaFree(h->d_conns); cudaFree(h->d_tile_counter);
   cudaFree(h->invvol); cudaFree(h->vol); cudaFree(h->srcvol); cudaFree(h->srcvol2);
   cudaFree(h->scratch_r); cudaFree(h->partials); cudaFree(h->d_norm); cudaFree(h->stage_buf);
-  cudaFree(h->adj_contrib); cudaFree(h->adj_lamg); cudaFree(h->adj_qx);
+  cudaFree(h->adj_prim); cudaFree(h->adj_cot); cudaFree(h->adj_lamg); cudaFree(h->adj_qx);
   cudaFree(h->d_bcs); cudaFree(h->d_bcmap);
   cudaFree(h->d_hsend); cudaFree(h->d_hrecv); cudaFree(h->d_hstiles); cudaFree(h->d_hrtiles); cudaFree(h->d_xtiles);
   cudaFree(h->geo_t);
@@ -1947,20 +1948,15 @@ int fv_adjoint_vjp(fv_handle hh, int stage, double dt, const double* qin_dev, co
   if (h->cfg.visc) return fail(h, FV_ERR_UNSUPPORTED, "the adjoint is built for the inviscid residual");
   cudaStream_t s = (cudaStream_t)stream;
   const int nd = h->cfg.dim;
-  // per-direction offsets of each block's faces in the contribution scratch
-  std::vector<long long> coff(3 * h->hb.size());
-  long long tot[3] = {0, 0, 0};
-  for (size_t b = 0; b < h->hb.size(); ++b) {
-    const FvBlockDev& B = h->hb[b];
-    for (int d = 0; d < 3; ++d) {
-      coff[3 * b + d] = tot[d];
-      if (d < nd) tot[d] += (long long)(B.ni + (d == 0)) * (B.nj + (d == 1)) * (B.nk + (d == 2));
-    }
+  long long nf_max = 0;
+  for (const FvBlockDev& B : h->hb) {
+    long long nf = 0;
+    for (int d = 0; d < nd; ++d) nf += (long long)(B.ni + (d == 0)) * (B.nj + (d == 1)) * (B.nk + (d == 2));
+    nf_max = std::max(nf_max, nf);
   }
-  const long long nfaces_all = tot[0] + tot[1] + tot[2];
-  if (!h->adj_contrib) CK(h, cudaMalloc(&h->adj_contrib, sizeof(double) * 20 * nfaces_all));
+  if (!h->adj_prim) CK(h, cudaMalloc(&h->adj_prim, sizeof(double) * h->state_elems));
+  if (!h->adj_cot) CK(h, cudaMalloc(&h->adj_cot, sizeof(double) * 10 * nf_max));
   if (!h->adj_lamg) CK(h, cudaMalloc(&h->adj_lamg, sizeof(double) * h->state_elems));
-  double* cdir[3] = {h->adj_contrib, h->adj_contrib + 20 * tot[0], h->adj_contrib + 20 * (tot[0] + tot[1])};
   // linearise around the state the forward stage saw: X(Q^(m-1)), ghosts exchanged
   const double* qx = qin_dev;
   if (h->conn_items || h->bc_items) {
@@ -1973,19 +1969,11 @@ int fv_adjoint_vjp(fv_handle hh, int stage, double dt, const double* qin_dev, co
   }
   const double alpha_dt = h->cfg.alpha[stage - 1] * dt;
   const FvStageArgs a = base_args(h);
-  for (size_t b = 0; b < h->hb.size(); ++b) {
-    const FvBlockDev& B = h->hb[b];
-    for (int d = 0; d < nd; ++d)
-      if (fv_adjoint_faces(B, d, qx, lam_out_dev, h->invvol, alpha_dt, (const double*)h->metric[d], h->nfaces[d],
-                           a.fp, h->adj_df64, cdir[d] + 20 * coff[3 * b + d], s))
-        return cuda_fail(h, cudaGetLastError(), "adjoint face kernel");
-  }
-  for (size_t b = 0; b < h->hb.size(); ++b) {
-    const FvBlockDev& B = h->hb[b];
-    if (fv_adjoint_gather(B, cdir[0] + 20 * coff[3 * b], cdir[1] + 20 * coff[3 * b + 1],
-                          nd == 3 ? cdir[2] + 20 * coff[3 * b + 2] : nullptr, nd == 3, h->adj_lamg, s))
-      return cuda_fail(h, cudaGetLastError(), "adjoint gather kernel");
-  }
+  const double* metric[3] = {(const double*)h->metric[0], (const double*)h->metric[1], (const double*)h->metric[2]};
+  for (const FvBlockDev& B : h->hb)
+    if (fv_adjoint_block(B, nd, qx, lam_out_dev, h->invvol, alpha_dt, metric, a.fp, h->adj_df64, h->adj_prim,
+                         h->adj_cot, h->adj_lamg, s))
+      return cuda_fail(h, cudaGetLastError(), "adjoint kernels");
   for (const FvConnDev& c : h->hconns)
     if (fv_adjoint_transpose(h->d_blocks, c, h->adj_lamg, s)) return cuda_fail(h, cudaGetLastError(), "adjoint transpose");
   for (const FvBlockDev& B : h->hb)

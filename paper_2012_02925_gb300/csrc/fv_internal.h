@@ -149,13 +149,13 @@ constexpr int FV_SHAPE_TABLE[FV_NUM_SHAPES][4] = {{32, 8, 256, 0}, {32, 4, 128, 
                                                   {32, 4, 128, 1}, {32, 7, 256, 0}, {32, 6, 256, 0},
                                                   {16, 12, 192, 0}, {16, 4, 128, 0}};
 
-// Discrete-adjoint kernels (fv_adjoint.cu): binary64 data; the face VJPs in
-// binary64 (double_float = 0) or double-float arithmetic.
-int fv_adjoint_faces(const FvBlockDev& B, int dir, const double* qin, const double* lam_out, const double* invvol,
-                     double alpha_dt, const double* metric, long long mstride, const FvFaceParams& fp,
-                     int double_float, double* contrib, cudaStream_t s);
-int fv_adjoint_gather(const FvBlockDev& B, const double* cx, const double* cy, const double* cz, int three_d,
-                      double* lamg, cudaStream_t s);
+// Discrete-adjoint kernels (fv_adjoint.cu): binary64 data; the sweeps in
+// binary64 (double_float = 0) or double-float arithmetic.  One block's ghosted
+// cotangent of its stage input into lamg; prim: 8 bytes per state entry of
+// every block, cot: 80 bytes per face of the block, scratch.
+int fv_adjoint_block(const FvBlockDev& B, int nd, const double* qin, const double* lam_out, const double* invvol,
+                     double alpha_dt, const double* const metric[3], const FvFaceParams& fp, int double_float,
+                     void* prim, void* cot, double* lamg, cudaStream_t s);
 int fv_adjoint_transpose(const FvBlockDev* d_blocks, const FvConnDev& c, double* lamg, cudaStream_t s);
 int fv_adjoint_finish(const FvBlockDev& B, const double* lamg, const double* lam_out, double* lam_in, double* lam_q0,
                       cudaStream_t s);
