@@ -116,13 +116,22 @@ __host__ __device__ constexpr bool stage_share() {
 }
 // planes in the 3-D ring: with shared slopes a pass reads planes k .. k+2
 // only, unless a slip-wall zeta face on a block's upper side reads k - 1
-template <class T, bool BC>
+// Two barriers a plane instead of three (DEEP): the plane after next is staged
+// beside the faces, and the next plane's slopes are taken beside the update,
+// which costs one more ring plane.  For the 64-cell tile, whose four resident
+// CTAs leave the room: 128^3 RK step 4.50 -> 4.42 ms, 64-block batch 26.6 ->
+// 25.3 ms.
+template <class T, int TX, int TY>
+__host__ __device__ constexpr bool stage_deep() {
+  return stage_share<T>() && TX * TY <= 64;
+}
+template <class T, int TX, int TY, bool BC>
 __host__ __device__ constexpr int stage_slots() {
-  return stage_share<T>() && !BC ? 3 : 4;
+  return (stage_share<T>() && !BC ? 3 : 4) + (stage_deep<T, TX, TY>() ? 1 : 0);
 }
 template <class T, int TX, int TY, bool FAST, bool VISC, bool BC>
 using StageSmemOf = StageSmem<T, TX, TY, (VISC && std::is_same<T, float>::value) ? 6 : 5,
-                              stage_share<T>(), stage_slots<T, BC>()>;
+                              stage_share<T>(), stage_slots<T, TX, TY, BC>()>;
 
 // resident CTAs per SM the register allocation must allow (shared memory
 // permits this many for the compiled shapes)
@@ -154,7 +163,8 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   constexpr int W = SM::W, PL = SM::PL;
   constexpr int NXI = SM::NXI, NETA = SM::NETA, NZETA = SM::NZETA;
   constexpr int NHX = SM::NHX, NHY = SM::NHY;
-  constexpr int NSLOT = DIM3 ? stage_slots<T, BC>() : 1;
+  constexpr int NSLOT = DIM3 ? stage_slots<T, TX, TY, BC>() : 1;
+  constexpr bool DEEP = DIM3 && stage_deep<T, TX, TY>();
   constexpr int NFACE = NXI + NETA + (DIM3 ? NZETA : 0);
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -168,7 +178,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   double* stg = reinterpret_cast<double*>(smem_raw + ((SM::typed(DIM3) + 15) / 16) * 16);  // [5][H][W] (PF)
   // ring slot of plane kk (kk >= -2)
   auto ring = [&](int kk) -> T* {
-    const int sl = NSLOT == 4 ? (kk & 3) : (NSLOT == 3 ? (kk + 6) % 3 : 0);
+    const int sl = NSLOT == 4 ? (kk & 3) : (NSLOT > 1 ? (kk + 2 * NSLOT) % NSLOT : 0);
     return Vs + sl * NV * PL;
   };
 
@@ -455,6 +465,11 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         // the zeta slope of plane k0-1; the first pass overwrites k0-2
         __syncthreads();
         slopes(k0 - 1, k0 - 1, false);
+        if constexpr (DEEP) {
+          load_plane(k0 + 1);
+          __syncthreads();
+          slopes(k0 - 1, k0, false);
+        }
         __syncthreads();
       }
     } else {
@@ -465,7 +480,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
     // In 3D the first pass (k = k0 - 1) evaluates only the zeta faces below
     // plane k0; every later pass is one plane.
     for (int k = DIM3 ? k0 - 1 : k0; k < k1; ++k) {
-      if (DIM3) {
+      if (DIM3 && !DEEP) {
         if (PF) {
           convert_staged(k + 2);
           __syncthreads();
@@ -476,7 +491,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         }
       }
       const T* P = ring(k);
-      if constexpr (SHARE) {
+      if constexpr (SHARE && !DEEP) {
         slopes(k, k + 1, !DIM3 || k >= k0);
         __syncthreads();
       }
@@ -572,8 +587,18 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         }
         do_face(s0, s1, s2, s3, hL, hR, hs, d, f, dp, dstr, code, side, vis);
       }
+      if constexpr (DEEP) {
+        // into the slot of plane k - 1 (with the wall overwrites of k - 2)
+        if (k + 3 <= k1 + 1) load_plane(k + 3);
+      }
       __syncthreads();
-      if (DIM3 && k < k0) continue;
+      if constexpr (DEEP) {
+        if (k + 1 < k1) slopes(k + 1, k + 2, true);
+      }
+      if (DIM3 && k < k0) {
+        if (DEEP) __syncthreads();
+        continue;
+      }
       // ---- per cell: flux differences in a fixed order, then the RK update ----
       for (int cc = tid; cc < TX * TY; cc += NT) {
         const int y = cc / TX, x = cc - y * TX;
@@ -669,6 +694,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
           }
         }
       }
+      if constexpr (DEEP) __syncthreads();   // the next pass's faces overwrite the fluxes
     }
     __syncthreads();   // smem is reused by the next tile
     if (tid == 0) s_next = (int)gridDim.x + atomicAdd(args.tile_counter, 1);
