@@ -165,13 +165,14 @@ typedef struct {
  *   dim: 2 (nk must be 1; no zeta fluxes) or 3.
  *   n_stages, alpha: Q^(m) = Q^(0) - alpha[m-1] dt / Omega R(Q^(m-1)),
  *     m = 1..n_stages (2..8).
- *   tile: 0 = automatic; else an index into the compiled tile shapes
+ *   tile: 0 = automatic (picked with the k-chunk from the blocks' extents);
+ *     else an index into the compiled tile shapes
  *     (1: 32x8 cells / 256 threads, 2: 32x4 / 128, 3: 16x8 / 128, 4: 30x8 / 256,
  *     5: 32x8 / 288, 6: 32x8 / 256 and 7: 32x4 / 128 with the next k-plane
  *     prefetched by cp.async - 6 and 7 for FV_PREC_FP32FLUX only -, 8: 32x7 / 256,
  *     9: 32x6 / 256, 10: 16x12 / 192, 11: 16x4 / 128).
  *   kchunk: k-planes per tile; 0 = automatic (about three tiles per resident
- *     CTA slot); -w = about w tiles per resident CTA slot.  Tiles are handed
+ *     CTA slot when the tile shape is given); -w = about w tiles per resident CTA slot.  Tiles are handed
  *     to persistent CTAs largest first through a device counter.
  *   flux: fv_flux (Roe by default); van Leer F+- split by the normal Mach
  *     number, Steger-Warming by the eigenvalues; F^ = F+(V_L) + F-(V_R).

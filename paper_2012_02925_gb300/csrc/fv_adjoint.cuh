@@ -1,11 +1,10 @@
 // Reverse-mode (vector-Jacobian) form of one face of the residual.
 //
-// The forward face is the one of fv_face.cuh: primitive recovery of the four
-// stencil cells (Section 2), MUSCL reconstruction with limiter, Eq. (flux) of
-// Section 7.2, and Roe's flux times the face area (Section 2).  Given the
-// cotangent Fbar of the face flux, face_vjp returns the cotangents of the 20
-// conserved inputs (4 cells x 5 variables).  Every intermediate of the forward
-// pass is recomputed and then swept backwards, statement by statement.
+// The forward face is the one of fv_face.cuh: MUSCL reconstruction with
+// limiter, Eq. (flux) of Section 7.2, and Roe's flux times the face area
+// (Section 2).  Given the cotangent of the face flux, roe_vjp returns the
+// cotangents of the two face states; lim_derivatives and prim_bwd transpose
+// the limiter and the primitive recovery (Section 2), once per cell.
 //
 // Written once for an arithmetic type T (fv_arith.cuh): binary64, or
 // double-float on the FP32 pipe (~48-bit significand; GB300's FP64 unit runs

@@ -2,11 +2,13 @@
 // around the fused stage kernel: metrics, ghost exchange, residual norms,
 // source scaling.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <map>
 #include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -32,6 +34,7 @@ struct fv_ctx {
   int ntiles = 0;
   int* d_tile_counter = nullptr;    // dynamic tile scheduling of the stage kernel
   FvLaunch launch{};
+  int kchunk = 0;                   // k-planes per tile as chosen (fv_config.kchunk's meaning)
   FxConsts fx{};                    // constants of the binary64 form's fixed-point Roe flux
   FvConnDev* d_conns = nullptr;
   long long conn_items = 0;
@@ -857,22 +860,69 @@ int copy_state(fv_ctx* h, const double* src, double* dst, bool to_internal, cuda
   return FV_OK;
 }
 
-void choose_launch(fv_ctx* h) {
-  const fv_config& c = h->cfg;
-  FvLaunch l{};
-  l.three_d = c.dim == 3;
-  int shape = c.tile;
-  if (shape <= 0) {
-    // automatic: narrow blocks prefer narrow tiles
-    int maxni = 0;
-    for (auto& b : h->hb) maxni = std::max(maxni, b.ni);
-    shape = maxni >= 24 ? 1 : 3;
-  }
+void set_shape(fv_ctx* h, int shape) {
+  FvLaunch& l = h->launch;
   shape = std::min(std::max(shape, 1), FV_NUM_SHAPES);
   l.shape = shape;
   l.tx = FV_SHAPE_TABLE[shape - 1][0];
   l.ty = FV_SHAPE_TABLE[shape - 1][1];
   l.threads = FV_SHAPE_TABLE[shape - 1][2];
+}
+
+// Resident CTAs per SM of the launch's kernel; a property of the kernel and
+// the device, asked of the driver once per process (a query of a few shapes
+// took 1 ms of each handle's creation)
+int query_occupancy(fv_ctx* h) {
+  static std::mutex lock;
+  static std::map<std::array<int, 7>, int> known;
+  const FvLaunch& l = h->launch;
+  const std::array<int, 7> key = {h->device, h->cfg.precision, l.shape, l.three_d, l.fast, l.visc, l.bc};
+  std::lock_guard<std::mutex> guard(lock);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  size_t smem = 0;
+  const int occ = stage_variant(h).occupancy(l, &smem);
+  if (occ > 0) known[key] = occ;
+  return occ;
+}
+
+long long columns_of(const FvBlockDev& b, const FvLaunch& l) {
+  return (long long)((b.ni + l.tx - 1) / l.tx) * ((b.nj + l.ty - 1) / l.ty);
+}
+
+// k-planes per tile of block b: kchunk > 0 as given, -w for about w tiles per
+// resident CTA slot, 0 for about three
+int kchunk_of(const FvBlockDev& b, int dim, int kchunk, long long slots, long long columns) {
+  if (dim == 2) return 1;
+  int kc = kchunk;
+  if (kc <= 0) {
+    const long long w = kc ? -(long long)kc : 3;
+    const long long want = std::max<long long>(1, kc ? w * slots / std::max<long long>(columns, 1)
+                                                       : (w * slots + columns - 1) / std::max<long long>(columns, 1));
+    kc = (int)std::max<long long>(kchunk ? 2 : 4, (b.nk + want - 1) / want);
+  }
+  return std::min(kc, b.nk);
+}
+
+// The launch's kernel (scheme, viscous and boundary variants) and tile shape.
+// Automatic shape and k-chunk (tile 0, kchunk 0): the pair with the smallest
+// estimated time among the shapes that were the fastest of some problem in
+// the form.  A tile takes its planes plus about 1.3 planes' worth of start-up
+// (halo planes, the first zeta faces).  A CTA's time is bound by its own
+// latencies: with `ref` resident CTAs (those of the measurement) or fewer a
+// tile-plane takes ref x cost x cells, and a wave of tiles the same whether
+// or not every slot has one; many more tiles than slots even out (dynamic
+// hand-out), up to half a tile at the end.  Costs per cell and plane:
+// measured RK steps of the 128^3 block and (2-D) of the 1100 x 300 inlet,
+// which fill the chip in every shape.  Measured on 15 problems from 1,024 to
+// 10.9 M cells, RK step with the fixed 32 x 8 shape (16 x 8 for narrow blocks)
+// over this rule's: binary64 1.2 .. 2.5, double-float 1.0 .. 2.2,
+// binary32 flux 1.0 .. 2.0; 64-block batch in binary64 39.3 -> 24.7 ms, in
+// binary32 flux 5.23 -> 4.74 ms.
+void choose_launch(fv_ctx* h) {
+  const fv_config& c = h->cfg;
+  FvLaunch l{};
+  l.three_d = c.dim == 3;
   l.fast = fv_default_scheme(c.flux, c.limiter, c.eps, c.kappa, c.harten, c.fix_all);
   // viscous kernels: the binary32 form fuses the viscous faces into the
   // stage kernel (its T on the fly costs a MUFU reciprocal); for binary64
@@ -882,34 +932,76 @@ void choose_launch(fv_ctx* h) {
   l.bc = 0;
   for (const FvBlockDev& b : h->hb) l.bc |= b.bcmap != nullptr;
   h->launch = l;
+  h->kchunk = c.kchunk;
+  if (c.tile > 0) {
+    set_shape(h, c.tile);
+    return;
+  }
+  struct Shape { int id, ref; double cost; };
+  static const Shape tables[2][3][6] = {
+      {{{11, 4, 4.42}, {9, 2, 4.33}, {3, 3, 4.51}},                                                // 3-D: binary64
+       {{1, 2, 2.73}, {8, 2, 2.75}, {9, 2, 2.97}, {11, 4, 3.87}},                                  // double-float
+       {{1, 4, 0.92}, {8, 4, 0.93}, {9, 4, 0.96}, {3, 7, 0.97}, {11, 8, 1.08}}},                   // binary32 flux
+      {{{11, 4, 5.75}, {9, 2, 5.26}, {3, 4, 4.67}, {8, 2, 4.81}},                                  // 2-D
+       {{1, 2, 3.56}, {8, 2, 3.38}, {9, 2, 3.76}, {3, 4, 3.64}, {11, 4, 4.40}},
+       {{1, 4, 1.29}, {8, 4, 1.27}, {9, 4, 1.35}, {3, 8, 1.28}, {11, 8, 1.51}}}};
+  const int form = c.precision == FV_PREC_FP64 ? 0 : (c.precision == FV_PREC_DF64 ? 1 : 2);
+  const Shape* table = tables[c.dim == 2][form];
+  static const int chunks[] = {0, -1, -2, 4, 8, 16, 32};
+  double best = 0.0;
+  int shape = 1, kchunk = c.kchunk;
+  for (const Shape* t = table; t->id; ++t) {
+    set_shape(h, t->id);
+    const int occ = query_occupancy(h);
+    if (occ <= 0) continue;
+    const FvLaunch& s = h->launch;
+    const long long slots = (long long)h->nsm * occ;
+    long long columns = 0;
+    for (const FvBlockDev& b : h->hb) columns += columns_of(b, s);
+    for (int kc0 : chunks) {
+      if (c.kchunk ? kc0 != chunks[0] : (c.dim == 2 && kc0 != 0)) continue;
+      const int want = c.kchunk ? c.kchunk : kc0;
+      const double start = c.dim == 3 ? 1.3 : 0.0;
+      double total = 0.0, longest = 0.0;
+      long long tiles = 0;
+      for (const FvBlockDev& b : h->hb) {
+        const int kc = kchunk_of(b, c.dim, want, slots, columns);
+        const long long n = columns_of(b, s), parts = (b.nk + kc - 1) / kc;
+        tiles += n * parts;
+        total += (double)n * (b.nk + parts * start);
+        longest = std::max(longest, kc + start);
+      }
+      const long long waves = (tiles + slots - 1) / slots;
+      double planes = total / (double)slots + 0.5 * longest;
+      // (binary32 flux, bound by throughput more than by latency: tiles of a
+      // wave drift apart, and a few long ones lose to many short ones)
+      if (waves <= 4) planes = std::min(waves * longest * (form == 2 ? 1.12 : 1.0), planes + 0.5 * longest);
+      // binary32 flux in 2-D: short tiles, and half-empty waves are quicker
+      if (form == 2 && c.dim == 2) planes = std::max(0.5, total / (double)slots) + 0.15;
+      const double time = planes * std::max(occ, t->ref) * t->cost * s.tx * s.ty;
+      if (best == 0.0 || time < best) {
+        best = time;
+        shape = t->id;
+        kchunk = want;
+      }
+    }
+  }
+  set_shape(h, shape);
+  h->kchunk = kchunk;
 }
-
-int query_occupancy(fv_ctx* h, size_t* smem) { return stage_variant(h).occupancy(h->launch, smem); }
 
 int build_tiles(fv_ctx* h) {
   const FvLaunch& l = h->launch;
-  size_t smem = 0;
-  const int occ = query_occupancy(h, &smem);
+  const int occ = query_occupancy(h);
   if (occ <= 0) return fail(h, FV_ERR_UNSUPPORTED, "stage kernel cannot be resident with this tile shape");
   const long long slots = (long long)h->nsm * occ;
   long long columns = 0;
-  for (auto& b : h->hb) columns += (long long)((b.ni + l.tx - 1) / l.tx) * ((b.nj + l.ty - 1) / l.ty);
+  for (auto& b : h->hb) columns += columns_of(b, l);
   std::vector<FvTile> tiles;
   std::vector<long long> cost;
   for (int bi = 0; bi < (int)h->hb.size(); ++bi) {
     const FvBlockDev& b = h->hb[bi];
-    int kc = h->cfg.kchunk;
-    if (h->cfg.dim == 2) kc = 1;
-    else if (kc == 0) {
-      // split k so that the whole problem fills the resident CTA slots a few times
-      const long long want = std::max<long long>(1, (3 * slots + columns - 1) / std::max<long long>(columns, 1));
-      kc = (int)std::max<long long>(4, (b.nk + want - 1) / want);
-    } else if (kc < 0) {
-      // -w: about w tiles per resident CTA slot
-      const long long want = std::max<long long>(1, (-kc * slots) / std::max<long long>(columns, 1));
-      kc = (int)std::max<long long>(2, (b.nk + want - 1) / want);
-    }
-    kc = std::min(kc, b.nk);
+    const int kc = kchunk_of(b, h->cfg.dim, h->kchunk, slots, columns);
     for (int k0 = 0; k0 < b.nk; k0 += kc)
       for (int j0 = 0; j0 < b.nj; j0 += l.ty)
         for (int i0 = 0; i0 < b.ni; i0 += l.tx) {
