@@ -4,15 +4,15 @@
 //   mu_c   = -alpha_m dt / Omega_c * lam_c              (cotangent of R_c)
 //   Fbar_f = mu_L(f) - mu_R(f)                          (R_L holds +F_f, R_R holds -F_f)
 //   per face: cotangents of its two states from Fbar_f    (roe_vjp)
-//   per cell: slopes and primitive recovery transposed    (adj_cell_kernel)
+//   per cell: slopes, then primitive recovery transposed  (adj_slope_kernel, adj_cell_kernel)
 //   ghost cotangents are added into their donor cells (transpose of X),
 //   fixed ghosts are constants.
 // Deterministic: the faces' cotangents go to a scratch array and every cell
 // gathers its own in a fixed order; connections are transposed one launch at
 // a time in table order.
 //
-// 96^3 VJP stage (van Albada), double-float sweeps 1.80 -> 0.98 ms, binary64
-// 4.58 -> 4.13 ms against one kernel per face that recovered its four cells'
+// 96^3 VJP stage (van Albada), double-float sweeps 1.80 -> 0.84 ms, binary64
+// 4.58 -> 2.77 ms against one kernel per face that recovered its four cells'
 // primitives, evaluated the limiter's derivatives (20 of them), and reversed
 // all of it into 20 conserved cotangents (12,700 instructions a face, 160
 // bytes written): a face now does its Roe part and writes 10 cotangents
@@ -145,30 +145,80 @@ __global__ void __launch_bounds__(NT, MINB) adj_face_kernel(const FvBlockDev B, 
   }
 }
 
-// Every ghosted cell's cotangent: per direction, the cell's own face states
-// V + h and V - h (h the limited half-slope of its forward difference a and
-// backward difference b) and its neighbours' slopes; then the primitive
-// recovery's transpose.  With Lb, Rb the cotangents of a cell's two face
-// states, alpha = dh/da (Lb - Rb) and beta = dh/db (Lb - Rb) (the unlimited
-// scheme's two slopes differ), the cell at p gets
-//   Lb + Rb - alpha(p) + beta(p) + alpha(p-1) - beta(p+1).
-// Fixed order of summation: xi, eta, zeta; deterministic.
+// The slopes of direction `dir`, transposed: cells m = -1 .. n_dir along it
+// (those with a face state), interior across it.  The cell's face states are
+// V + h and V - h with h the limited half-slope of its forward difference a
+// and backward difference b.  With L, R the cotangents of the two (zero where
+// the face does not exist), alpha = dh/da (L - R) and beta = dh/db (L - R)
+// (the unlimited scheme's two slopes differ), the cell itself gets
+// L + R - alpha + beta, the next one alpha, the one before -beta: stored
+// component by component, one evaluation per cell, direction and variable
+// (evaluated three times, by each cell that takes a share, the 96^3 VJP stage
+// took 0.98 instead of 0.84 ms in double-float, 4.13 instead of 2.77 in binary64).
 template <class T>
-__global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const typename AdjMem<T>::type* __restrict__ prim,
-                                                       const typename AdjMem<T>::type* __restrict__ cx,
-                                                       const typename AdjMem<T>::type* __restrict__ cy,
-                                                       const typename AdjMem<T>::type* __restrict__ cz, int three_d,
-                                                       const AdjParams PP, double* __restrict__ lamg) {
+__global__ void __launch_bounds__(128) adj_slope_kernel(const FvBlockDev B, int dir,
+                                                        const typename AdjMem<T>::type* __restrict__ prim,
+                                                        const typename AdjMem<T>::type* __restrict__ cot,
+                                                        const AdjParams PP, typename AdjMem<T>::type* __restrict__ out) {
   using S = Sc<T>;
   using M = AdjMem<T>;
   const AdjC<T> P = adj_consts<T>(PP);
-  const int gi = B.ni + 2 * FV_GHOST, gj = B.nj + 2 * FV_GHOST, gk = B.nk + 2 * FV_GHOST;
+  const int ei = B.ni + (dir == 0), ej = B.nj + (dir == 1), ek = B.nk + (dir == 2);
+  const int ci = B.ni + 2 * (dir == 0), cj = B.nj + 2 * (dir == 1), ck = B.nk + 2 * (dir == 2);
+  const long long nf = (long long)ei * ej * ek, nc = (long long)ci * cj * ck;
+  const long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (x >= nc) return;
+  const int i = (int)(x % ci) - (dir == 0), j = (int)((x / ci) % cj) - (dir == 1), k = (int)(x / ((long long)ci * cj)) - (dir == 2);
+  const int m = dir == 0 ? i : (dir == 1 ? j : k), n_dir = dir == 0 ? B.ni : (dir == 1 ? B.nj : B.nk);
+  const long long st = dir == 0 ? 1 : (dir == 1 ? B.jstride : B.kstride);
+  const long long fs = dir == 0 ? 1 : (dir == 1 ? ei : (long long)ei * ej);
+  const long long f = ((long long)k * ej + j) * ei + i;          // the cell's lower face
+  const typename M::type* v = prim + B.qoff + ghost_index(B, i, j, k);
+#pragma unroll 1
+  for (int q = 0; q < 5; ++q) {
+    const T L = m < n_dir ? M::ld(cot + q * nf + f + fs) : S::c(0.0);
+    const T R = m >= 0 ? M::ld(cot + (5 + q) * nf + f) : S::c(0.0);
+    const T vm = M::ld(v + q * B.plane - st), v0 = M::ld(v + q * B.plane), vp = M::ld(v + q * B.plane + st);
+    T al, be;
+    if (P.limiter != 0) {
+      T da, db;
+      lim_derivatives(P, vp - v0, v0 - vm, da, db);
+      const T d = P.e2 * (L - R);
+      al = d * da;
+      be = d * db;
+    } else {
+      al = P.e4kp * L - P.e4km * R;
+      be = P.e4km * L - P.e4kp * R;
+    }
+    M::st(out + q * nc + x, (L + R) - (al - be));
+    M::st(out + (5 + q) * nc + x, al);
+    M::st(out + (10 + q) * nc + x, be);
+  }
+}
+
+// The cells' cotangents: the slope kernel's shares in a fixed order (xi, eta,
+// zeta; deterministic) and the primitive recovery's transpose.  Into lamg for
+// every ghosted cell; or, when no connection has to be transposed (lam_in not
+// null), straight to lam_in for the interior cells, with lam_q0 += lam_out.
+template <class T>
+__global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const typename AdjMem<T>::type* __restrict__ prim,
+                                                       const typename AdjMem<T>::type* __restrict__ sx,
+                                                       const typename AdjMem<T>::type* __restrict__ sy,
+                                                       const typename AdjMem<T>::type* __restrict__ sz, int three_d,
+                                                       const AdjParams PP, double* __restrict__ lamg,
+                                                       const double* __restrict__ lam_out, double* __restrict__ lam_in,
+                                                       double* __restrict__ lam_q0) {
+  using S = Sc<T>;
+  using M = AdjMem<T>;
+  const AdjC<T> P = adj_consts<T>(PP);
+  const int g = lam_in ? 0 : FV_GHOST;
+  const int gi = B.ni + 2 * g, gj = B.nj + 2 * g, gk = B.nk + 2 * g;
   const long long n = (long long)gi * gj * gk;
   const long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (x >= n) return;
-  const int i = (int)(x % gi) - FV_GHOST, j = (int)((x / gi) % gj) - FV_GHOST, k = (int)(x / ((long long)gi * gj)) - FV_GHOST;
+  const int i = (int)(x % gi) - g, j = (int)((x / gi) % gj) - g, k = (int)(x / ((long long)gi * gj)) - g;
   const bool ii = i >= 0 && i < B.ni, jj = j >= 0 && j < B.nj, kk = k >= 0 && k < B.nk;
-  const typename M::type* v = prim + B.qoff + x;
+  const long long gx = B.qoff + ghost_index(B, i, j, k);
   T Vb[5];
 #pragma unroll
   for (int m = 0; m < 5; ++m) Vb[m] = S::c(0.0);
@@ -176,42 +226,20 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const
   for (int dir = 0; dir < 2 + three_d; ++dir) {
     if (!(dir == 0 ? jj && kk : (dir == 1 ? ii && kk : ii && jj))) continue;
     const int p = dir == 0 ? i : (dir == 1 ? j : k), nd = dir == 0 ? B.ni : (dir == 1 ? B.nj : B.nk);
-    const long long st = dir == 0 ? 1 : (dir == 1 ? B.jstride : B.kstride);
-    const typename M::type* c = dir == 0 ? cx : (dir == 1 ? cy : cz);
-    // face g = p's index, and the distance of two faces along the direction
-    const long long ei = B.ni + (dir == 0), ej = B.nj + (dir == 1), ek = B.nk + (dir == 2);
-    const long long nf = ei * ej * ek, fs = dir == 0 ? 1 : (dir == 1 ? ei : ei * ej);
-    const long long f0 = ((long long)k * ej + j) * ei + i;
-    // cells p-1, p, p+1 with a face state: -1 .. nd
+    const typename M::type* s = dir == 0 ? sx : (dir == 1 ? sy : sz);
+    const long long ci = B.ni + 2 * (dir == 0), cj = B.nj + 2 * (dir == 1), ck = B.nk + 2 * (dir == 2);
+    const long long nc = ci * cj * ck, st = dir == 0 ? 1 : (dir == 1 ? ci : ci * cj);
+    const long long c = ((long long)(k + (dir == 2)) * cj + (j + (dir == 1))) * ci + (i + (dir == 0));
+    const bool own = p >= -1 && p <= nd, lo = p >= 0 && p <= nd + 1, up = p >= -2 && p <= nd - 1;
 #pragma unroll
-    for (int o = -1; o <= 1; ++o) {
-      const int m = p + o;
-      if (m < -1 || m > nd) continue;
-      const bool up = m + 1 <= nd, lo = m >= 0;                 // its upper and lower face exist
-#pragma unroll 1
-      for (int q = 0; q < 5; ++q) {
-        const T L = up ? M::ld(c + q * nf + f0 + (o + 1) * fs) : S::c(0.0);
-        const T R = lo ? M::ld(c + (5 + q) * nf + f0 + o * fs) : S::c(0.0);
-        const typename M::type* w = v + q * B.plane + o * st;
-        const T vm = M::ld(w - st), v0 = M::ld(w), vp = M::ld(w + st);
-        T al, be;
-        if (P.limiter != 0) {
-          T da, db;
-          lim_derivatives(P, vp - v0, v0 - vm, da, db);
-          const T d = P.e2 * (L - R);
-          al = d * da;
-          be = d * db;
-        } else {
-          al = P.e4kp * L - P.e4km * R;
-          be = P.e4km * L - P.e4kp * R;
-        }
-        const T add = o == 0 ? (L + R) - (al - be) : (o < 0 ? al : -be);
-#pragma unroll
-        for (int z = 0; z < 5; ++z) Vb[z] = z == q ? Vb[z] + add : Vb[z];
-      }
+    for (int q = 0; q < 5; ++q) {
+      if (own) Vb[q] = Vb[q] + M::ld(s + q * nc + c);
+      if (lo) Vb[q] = Vb[q] + M::ld(s + (5 + q) * nc + c - st);
+      if (up) Vb[q] = Vb[q] - M::ld(s + (10 + q) * nc + c + st);
     }
   }
   // the cell's primitives and the transpose of the recovery
+  const typename M::type* v = prim + gx;
   PrimFwd<T> s;
   s.r = M::ld(v);
   s.u = M::ld(v + B.plane);
@@ -221,10 +249,18 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const
   s.k = S::dot3(s.u, s.u, s.v, s.v, s.w, s.w);
   T qb[5];
   prim_bwd(P, s, Vb, qb);
-  double* o = lamg + B.qoff + x;
-  const bool any = (ii && jj) || (ii && kk) || (jj && kk);
+  if (lam_in) {
+    const long long o = 5 * B.cell_off + x;
 #pragma unroll
-  for (int m = 0; m < 5; ++m) o[m * B.plane] = any ? S::to_d(qb[m]) : 0.0;
+    for (int m = 0; m < 5; ++m) {
+      lam_in[o + m * n] = S::to_d(qb[m]);
+      lam_q0[o + m * n] += lam_out[o + m * n];
+    }
+  } else {
+    const bool any = (ii && jj) || (ii && kk) || (jj && kk);
+#pragma unroll
+    for (int m = 0; m < 5; ++m) lamg[gx + m * B.plane] = any ? S::to_d(qb[m]) : 0.0;
+  }
 }
 
 // transpose of one connection: donor interior cell += ghost cotangent
@@ -299,32 +335,36 @@ AdjParams adj_params(const FvFaceParams& fp) {
 template <class T, int MINB>
 int adjoint_block(const FvBlockDev& B, int nd, const double* qin, const double* lam_out, const double* invvol,
                   double alpha_dt, const double* const metric[3], const FvFaceParams& fp, void* prim_mem, void* cot_mem,
-                  double* lamg, cudaStream_t s) {
+                  void* slope_mem, double* lamg, double* lam_in, double* lam_q0, cudaStream_t s) {
   using MT = typename AdjMem<T>::type;
   const AdjParams P = adj_params(fp);
   MT* prim = static_cast<MT*>(prim_mem);
+  MT* cot = static_cast<MT*>(cot_mem);
   adj_prim_kernel<T><<<grid_of(B.plane, 256), 256, 0, s>>>(B, qin, P, prim);
-  MT* c[3] = {static_cast<MT*>(cot_mem), nullptr, nullptr};
+  MT* sl[3] = {static_cast<MT*>(slope_mem), nullptr, nullptr};
   for (int d = 0; d < nd; ++d) {
     const long long nf = (long long)(B.ni + (d == 0)) * (B.nj + (d == 1)) * (B.nk + (d == 2));
-    if (d) {
-      const long long before = (long long)(B.ni + (d == 1)) * (B.nj + (d == 2)) * B.nk;
-      c[d] = c[d - 1] + 10 * before;
-    }
+    const long long nc = (long long)(B.ni + 2 * (d == 0)) * (B.nj + 2 * (d == 1)) * (B.nk + 2 * (d == 2));
     adj_face_kernel<T, 128, MINB><<<(unsigned)((nf + 127) / 128), 128, 0, s>>>(B, d, prim, lam_out, invvol, alpha_dt,
-                                                                             metric[d], P, c[d]);
+                                                                             metric[d], P, cot);
+    adj_slope_kernel<T><<<(unsigned)((nc + 127) / 128), 128, 0, s>>>(B, d, prim, cot, P, sl[d]);
+    if (d < 2) sl[d + 1] = sl[d] + 15 * nc;
   }
-  const long long n = (long long)(B.ni + 4) * (B.nj + 4) * (B.nk + 4);
-  adj_cell_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(B, prim, c[0], c[1], c[2], nd == 3, P, lamg);
+  const int g = lam_in ? 0 : FV_GHOST;
+  const long long n = (long long)(B.ni + 2 * g) * (B.nj + 2 * g) * (B.nk + 2 * g);
+  adj_cell_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(B, prim, sl[0], sl[1], sl[2], nd == 3, P, lamg, lam_out,
+                                                               lam_in, lam_q0);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 }  // namespace
 
 int fv_adjoint_block(const FvBlockDev& B, int nd, const double* qin, const double* lam_out, const double* invvol,
                      double alpha_dt, const double* const metric[3], const FvFaceParams& fp, int double_float,
-                     void* prim, void* cot, double* lamg, cudaStream_t s) {
-  return double_float ? adjoint_block<df64, 4>(B, nd, qin, lam_out, invvol, alpha_dt, metric, fp, prim, cot, lamg, s)
-                      : adjoint_block<double, 3>(B, nd, qin, lam_out, invvol, alpha_dt, metric, fp, prim, cot, lamg, s);
+                     void* prim, void* cot, void* slopes, double* lamg, double* lam_in, double* lam_q0, cudaStream_t s) {
+  return double_float ? adjoint_block<df64, 4>(B, nd, qin, lam_out, invvol, alpha_dt, metric, fp, prim, cot, slopes, lamg,
+                                               lam_in, lam_q0, s)
+                      : adjoint_block<double, 3>(B, nd, qin, lam_out, invvol, alpha_dt, metric, fp, prim, cot, slopes,
+                                                 lamg, lam_in, lam_q0, s);
 }
 
 int fv_adjoint_transpose(const FvBlockDev* d_blocks, const FvConnDev& c, double* lamg, cudaStream_t s) {

@@ -56,7 +56,8 @@ struct fv_ctx {
   double* partials = nullptr;       // per-CTA norm partials
   double* d_norm = nullptr;         // 11 doubles
   double* adj_prim = nullptr;       // adjoint: primitive variables of the stage input
-  double* adj_cot = nullptr;        // adjoint: cotangents of the face states, one block at a time (10 per face)
+  double* adj_cot = nullptr;        // adjoint: cotangents of the face states, one block and direction at a time (10 per face)
+  double* adj_slope = nullptr;      // adjoint: the slopes' shares, one block at a time (15 per cell and direction)
   double* adj_lamg = nullptr;       // adjoint: ghosted cotangent of Q^(m-1)
   double* adj_qx = nullptr;         // adjoint: X(Q^(m-1)), the exchanged stage input
   int adj_df64 = 0;                 // adjoint face VJPs in double-float arithmetic (fv_set_adjoint_arith)
@@ -1481,7 +1482,7 @@ int fv_destroy(fv_handle hh) {
   cudaFree(h->d_blocks); cudaFree(h->d_tiles); cudaFree(h->d_conns); cudaFree(h->d_tile_counter);
   cudaFree(h->invvol); cudaFree(h->vol); cudaFree(h->srcvol); cudaFree(h->srcvol2);
   cudaFree(h->scratch_r); cudaFree(h->partials); cudaFree(h->d_norm); cudaFree(h->stage_buf);
-  cudaFree(h->adj_prim); cudaFree(h->adj_cot); cudaFree(h->adj_lamg); cudaFree(h->adj_qx);
+  cudaFree(h->adj_prim); cudaFree(h->adj_cot); cudaFree(h->adj_slope); cudaFree(h->adj_lamg); cudaFree(h->adj_qx);
   cudaFree(h->d_bcs); cudaFree(h->d_bcmap);
   cudaFree(h->d_hsend); cudaFree(h->d_hrecv); cudaFree(h->d_hstiles); cudaFree(h->d_hrtiles); cudaFree(h->d_xtiles);
   cudaFree(h->geo_t);
@@ -2040,15 +2041,21 @@ int fv_adjoint_vjp(fv_handle hh, int stage, double dt, const double* qin_dev, co
   if (h->cfg.visc) return fail(h, FV_ERR_UNSUPPORTED, "the adjoint is built for the inviscid residual");
   cudaStream_t s = (cudaStream_t)stream;
   const int nd = h->cfg.dim;
-  long long nf_max = 0;
+  long long nf_max = 0, nc_max = 0;
   for (const FvBlockDev& B : h->hb) {
-    long long nf = 0;
-    for (int d = 0; d < nd; ++d) nf += (long long)(B.ni + (d == 0)) * (B.nj + (d == 1)) * (B.nk + (d == 2));
-    nf_max = std::max(nf_max, nf);
+    long long nc = 0;
+    for (int d = 0; d < nd; ++d) {
+      nf_max = std::max(nf_max, (long long)(B.ni + (d == 0)) * (B.nj + (d == 1)) * (B.nk + (d == 2)));
+      nc += (long long)(B.ni + 2 * (d == 0)) * (B.nj + 2 * (d == 1)) * (B.nk + 2 * (d == 2));
+    }
+    nc_max = std::max(nc_max, nc);
   }
   if (!h->adj_prim) CK(h, cudaMalloc(&h->adj_prim, sizeof(double) * h->state_elems));
   if (!h->adj_cot) CK(h, cudaMalloc(&h->adj_cot, sizeof(double) * 10 * nf_max));
-  if (!h->adj_lamg) CK(h, cudaMalloc(&h->adj_lamg, sizeof(double) * h->state_elems));
+  if (!h->adj_slope) CK(h, cudaMalloc(&h->adj_slope, sizeof(double) * 15 * nc_max));
+  // connections to transpose: through the ghosted cotangent
+  const bool ghosted = !h->hconns.empty();
+  if (ghosted && !h->adj_lamg) CK(h, cudaMalloc(&h->adj_lamg, sizeof(double) * h->state_elems));
   // linearise around the state the forward stage saw: X(Q^(m-1)), ghosts exchanged
   const double* qx = qin_dev;
   if (h->conn_items || h->bc_items) {
@@ -2064,8 +2071,9 @@ int fv_adjoint_vjp(fv_handle hh, int stage, double dt, const double* qin_dev, co
   const double* metric[3] = {(const double*)h->metric[0], (const double*)h->metric[1], (const double*)h->metric[2]};
   for (const FvBlockDev& B : h->hb)
     if (fv_adjoint_block(B, nd, qx, lam_out_dev, h->invvol, alpha_dt, metric, a.fp, h->adj_df64, h->adj_prim,
-                         h->adj_cot, h->adj_lamg, s))
+                         h->adj_cot, h->adj_slope, h->adj_lamg, ghosted ? nullptr : lam_in_dev, lam_q0_dev, s))
       return cuda_fail(h, cudaGetLastError(), "adjoint kernels");
+  if (!ghosted) return FV_OK;
   for (const FvConnDev& c : h->hconns)
     if (fv_adjoint_transpose(h->d_blocks, c, h->adj_lamg, s)) return cuda_fail(h, cudaGetLastError(), "adjoint transpose");
   for (const FvBlockDev& B : h->hb)

@@ -150,12 +150,15 @@ constexpr int FV_SHAPE_TABLE[FV_NUM_SHAPES][4] = {{32, 8, 256, 0}, {32, 4, 128, 
                                                   {16, 12, 192, 0}, {16, 4, 128, 0}};
 
 // Discrete-adjoint kernels (fv_adjoint.cu): binary64 data; the sweeps in
-// binary64 (double_float = 0) or double-float arithmetic.  One block's ghosted
-// cotangent of its stage input into lamg; prim: 8 bytes per state entry of
-// every block, cot: 80 bytes per face of the block, scratch.
+// binary64 (double_float = 0) or double-float arithmetic.  One block's cotangent
+// of its stage input: into lamg, ghosted, or (lam_in not null) the interior
+// into lam_in with lam_q0 += lam_out.  Scratch, reused by every block in stream
+// order: prim 8 bytes per state entry of every block, cot 80 bytes per face of
+// the block's largest direction, slopes 120 bytes per cell and direction (two
+// cells longer along it).
 int fv_adjoint_block(const FvBlockDev& B, int nd, const double* qin, const double* lam_out, const double* invvol,
                      double alpha_dt, const double* const metric[3], const FvFaceParams& fp, int double_float,
-                     void* prim, void* cot, double* lamg, cudaStream_t s);
+                     void* prim, void* cot, void* slopes, double* lamg, double* lam_in, double* lam_q0, cudaStream_t s);
 int fv_adjoint_transpose(const FvBlockDev* d_blocks, const FvConnDev& c, double* lamg, cudaStream_t s);
 int fv_adjoint_finish(const FvBlockDev& B, const double* lamg, const double* lam_out, double* lam_in, double* lam_q0,
                       cudaStream_t s);
