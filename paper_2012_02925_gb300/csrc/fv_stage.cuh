@@ -744,7 +744,10 @@ static int occupancy_t(bool three_d, size_t* smem_out) {
 // Compiled tile shapes (TX, TY, threads, prefetch); the shape ids of
 // fv_config.tile are 1-based indices into this list.  The prefetching shapes
 // are built for the binary32-flux form only (their staging plane would cost
-// the wider forms a resident CTA).
+// the wider forms a resident CTA), the square 64-cell one for binary64 only
+// (fewer halo cells, faces and slopes than 16 x 4: 64-block batch 25.3 -> 24.0
+// ms, 128^3 4.42 -> 4.35 ms in that shape; its rows of 64 bytes do not matter
+// to a kernel at 6 % of the memory bandwidth).
 #define FV_SHAPES(X)      \
   X(1, 32, 8, 256, false) \
   X(2, 32, 4, 128, false) \
@@ -756,17 +759,18 @@ static int occupancy_t(bool three_d, size_t* smem_out) {
   X(8, 32, 7, 256, false) \
   X(9, 32, 6, 256, false) \
   X(10, 16, 12, 192, false) \
-  X(11, 16, 4, 128, false)
+  X(11, 16, 4, 128, false) \
+  X(12, 8, 8, 128, false)
 
 // FAST selects the compile-time default scheme (FaceCFast); each
 // translation unit instantiates one combination of FAST, VISC and BC.
 template <class T, bool FAST, bool VISC, bool BC>
 int fv_dispatch_launch(const FvStageArgs& a, const FvLaunch& l, cudaStream_t s) {
-  constexpr bool allow_pf = std::is_same<T, float>::value;
+  constexpr bool allow_pf = std::is_same<T, float>::value, wide = std::is_same<T, double>::value;
 #define FV_LAUNCH_CASE(ID, TX, TY, NT, PF)                                     \
   if (l.shape == ID) {                                                          \
-    if (PF && !allow_pf) return -2;                                             \
-    return launch_stage_t<T, TX, TY, NT, PF && allow_pf, FAST, VISC, BC>(a, l, s); \
+    if ((PF && !allow_pf) || (ID == 12 && !wide)) return -2;                    \
+    return launch_stage_t<T, ID == 12 && !wide ? 16 : TX, ID == 12 && !wide ? 4 : TY, NT, PF && allow_pf, FAST, VISC, BC>(a, l, s); \
   }
   FV_SHAPES(FV_LAUNCH_CASE)
 #undef FV_LAUNCH_CASE
@@ -775,12 +779,12 @@ int fv_dispatch_launch(const FvStageArgs& a, const FvLaunch& l, cudaStream_t s) 
 
 template <class T, bool FAST, bool VISC, bool BC>
 int fv_dispatch_occupancy(const FvLaunch& l, size_t* smem) {
-  constexpr bool allow_pf = std::is_same<T, float>::value;
+  constexpr bool allow_pf = std::is_same<T, float>::value, wide = std::is_same<T, double>::value;
   const bool d3 = l.three_d != 0;
 #define FV_OCC_CASE(ID, TX, TY, NT, PF)                                         \
   if (l.shape == ID) {                                                          \
-    if (PF && !allow_pf) return 0;                                              \
-    return occupancy_t<T, TX, TY, NT, PF && allow_pf, FAST, VISC, BC>(d3, smem); \
+    if ((PF && !allow_pf) || (ID == 12 && !wide)) return 0;                     \
+    return occupancy_t<T, ID == 12 && !wide ? 16 : TX, ID == 12 && !wide ? 4 : TY, NT, PF && allow_pf, FAST, VISC, BC>(d3, smem); \
   }
   FV_SHAPES(FV_OCC_CASE)
 #undef FV_OCC_CASE

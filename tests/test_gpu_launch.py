@@ -26,7 +26,7 @@ def test_bit_equal_to_a_given_tile(name, prec):
     import paper_2012_02925_gb300 as fv
     pb = PROBLEMS[name]()
     out = []
-    for tile, kchunk in ((0, 0), (3, 2), (11, 5)):
+    for tile, kchunk in ((0, 0), (3, 2), (11, 5)) + (((12, 3),) if prec == "fp64" else ()):
         s = fv.Solver.from_problem(pb, precision=prec, tile=tile, kchunk=kchunk)
         s.set_state(torch.from_numpy(pb.q).cuda())
         if pb.source is not None:
@@ -36,4 +36,4 @@ def test_bit_equal_to_a_given_tile(name, prec):
         out.append(s.get_state(0).cpu().numpy())
         s.close()
     assert np.isfinite(out[0]).all()
-    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+    assert all(np.array_equal(out[0], x) for x in out[1:])
