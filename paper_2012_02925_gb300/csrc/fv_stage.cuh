@@ -27,9 +27,9 @@ template <class T> struct MetricStore;
 template <> struct MetricStore<double> {
   using type = double;
   static __device__ __forceinline__ double ld(const double* p, long long i) { return __ldg(p + i); }
-  static __device__ __forceinline__ void ld4(const double* p, long long f, double& a, double& b, double& c,
+  static __device__ __forceinline__ void ld4(const double* p, unsigned f, double& a, double& b, double& c,
                                              double& d) {
-    const double2* q = reinterpret_cast<const double2*>(p + 4 * f);
+    const double2* q = reinterpret_cast<const double2*>(p) + 2ull * f;
     const double2 x = __ldg(q), y = __ldg(q + 1);
     a = x.x; b = x.y; c = y.x; d = y.y;
   }
@@ -40,8 +40,8 @@ template <> struct MetricStore<df64> {
     float2 v = __ldg(p + i);
     return mk(v.x, v.y);
   }
-  static __device__ __forceinline__ void ld4(const float2* p, long long f, df64& a, df64& b, df64& c, df64& d) {
-    const float4* q = reinterpret_cast<const float4*>(p + 4 * f);
+  static __device__ __forceinline__ void ld4(const float2* p, unsigned f, df64& a, df64& b, df64& c, df64& d) {
+    const float4* q = reinterpret_cast<const float4*>(p) + 2ull * f;
     const float4 x = __ldg(q), y = __ldg(q + 1);
     a = mk(x.x, x.y); b = mk(x.z, x.w); c = mk(y.x, y.y); d = mk(y.z, y.w);
   }
@@ -49,8 +49,8 @@ template <> struct MetricStore<df64> {
 template <> struct MetricStore<float> {
   using type = float;
   static __device__ __forceinline__ float ld(const float* p, long long i) { return __ldg(p + i); }
-  static __device__ __forceinline__ void ld4(const float* p, long long f, float& a, float& b, float& c, float& d) {
-    const float4 x = __ldg(reinterpret_cast<const float4*>(p + 4 * f));
+  static __device__ __forceinline__ void ld4(const float* p, unsigned f, float& a, float& b, float& c, float& d) {
+    const float4 x = __ldg(reinterpret_cast<const float4*>(p) + f);
     a = x.x; b = x.y; c = x.z; d = x.w;
   }
 };
@@ -133,6 +133,19 @@ template <class T, int TX, int TY, bool FAST, bool VISC, bool BC>
 using StageSmemOf = StageSmem<T, TX, TY, (VISC && std::is_same<T, float>::value) ? 6 : 5,
                               stage_share<T>(), stage_slots<T, TX, TY, BC>()>;
 
+// Face items by rows: with a warp per row of 32 cells and one more for the
+// edges, round r of a plane is direction r - warp y takes the faces below row
+// y's cells, the last warp the TY faces after the rows (xi) and the TX faces
+// above the last row (eta) - so an item needs no decoding.  Same number of
+// rounds as the balanced list of the same shape.  128^3 RK step, 32 x 7 tile:
+// double-float 2.77 -> 2.46 ms, binary32 flux 0.854 -> 0.745 ms, of which the
+// block constants in shared memory (below) 4 and 9 %, as in the listed shapes.
+// (Not for the fused viscous faces, whose work hides the decoding.)
+template <int TX, int TY, int NT>
+__host__ __device__ constexpr bool stage_rows() {
+  return TX == 32 && NT == 32 * (TY + 1);
+}
+
 // resident CTAs per SM the register allocation must allow (shared memory
 // permits this many for the compiled shapes)
 template <class T, int NT, bool VISC>
@@ -166,6 +179,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   constexpr int NSLOT = DIM3 ? stage_slots<T, TX, TY, BC>() : 1;
   constexpr bool DEEP = DIM3 && stage_deep<T, TX, TY>();
   constexpr int NFACE = NXI + NETA + (DIM3 ? NZETA : 0);
+  constexpr bool ROWS = !FUSED_VISC && stage_rows<TX, TY, NT>();
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* Vs = reinterpret_cast<T*>(smem_raw);        // [NSLOT][NV][H][W]
@@ -186,9 +200,14 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   const CC C = CC::from(make_face_consts<T>(args.fp));
   const ViscC<T> VK = make_visc_consts<T>(args.vp);
   const typename VGeo<T>::type* geo = reinterpret_cast<const typename VGeo<T>::type*>(args.geo);
-  const MT* mxi = reinterpret_cast<const MT*>(args.metric[0]);
-  const MT* meta = reinterpret_cast<const MT*>(args.metric[1]);
-  const MT* mzeta = reinterpret_cast<const MT*>(args.metric[2]);
+  // The tile's block constants as the faces read them: the face records of
+  // each direction (metrics, viscous fluxes), or the Cartesian unit normals
+  // and areas, converted once a tile (read from the block's record at each
+  // face, with the conversions: 64-block batch in binary32 flux 4.8 against
+  // 4.4 ms, 256x256x128 periodic block in double-float 11.0 against 9.8 ms).
+  __shared__ const MT* s_met[3];
+  __shared__ const MT* s_vis[3];
+  __shared__ __align__(16) T s_cart[12];
 
   // Tiles 0..gridDim-1 go to the CTAs in order; later ones are handed out
   // dynamically (largest first, as the table is sorted) through a counter
@@ -202,6 +221,17 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
     const long long js = B.jstride, ks = B.kstride, pl = B.plane;
     const double* qin = args.qin + B.qoff;
     const bool cart = B.cartesian != 0;
+    // the block's boundary codes, for the tiles that have a face on its surface
+    const signed char* bcmap = nullptr;
+    if (BC && (i0 == 0 || j0 == 0 || i0 + TX >= ni || j0 + TY >= nj || (DIM3 && (k0 == 0 || k1 == nk)))) bcmap = B.bcmap;
+    if (tid < 3) {
+      s_met[tid] = reinterpret_cast<const MT*>(args.metric[tid]) + 4 * B.face_off[tid];
+      if (VISC_PAIRS) s_vis[tid] = reinterpret_cast<const MT*>(args.fv[tid]) + 4 * B.vface_off[tid];
+    }
+    if (cart && tid < 12) {
+      const int d = tid >> 2, x = tid & 3;
+      s_cart[tid] = S::from_d(x < 3 ? B.cart_n[d][x] : B.cart_area[d]);
+    }
 
     // Per-thread work descriptors, fixed for the whole tile (only the plane
     // index changes along k): the halo cells this thread stages ...
@@ -308,14 +338,13 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
     };
     // hL, hR, hs (SHARE): the half-slopes of s1 and s2, components hs apart
     auto do_face = [&](const T* s0, const T* s1, const T* s2, const T* s3, const T* hL, const T* hR, int hs,
-                       int dir, long long f, T* dst, int dstr, int code, int side, const VisArgs& vis) {
+                       int dir, unsigned f, T* dst, int dstr, int code, int side, const VisArgs& vis) {
       T nx, ny, nz, A;
       if (cart) {
-        nx = S::from_d(B.cart_n[dir][0]); ny = S::from_d(B.cart_n[dir][1]);
-        nz = S::from_d(B.cart_n[dir][2]); A = S::from_d(B.cart_area[dir]);
+        const T* c = s_cart + 4 * dir;
+        nx = c[0]; ny = c[1]; nz = c[2]; A = c[3];
       } else {
-        const MT* m = dir == 0 ? mxi : (dir == 1 ? meta : mzeta);
-        MetricStore<T>::ld4(m, f, nx, ny, nz, A);
+        MetricStore<T>::ld4(s_met[dir], f, nx, ny, nz, A);
       }
       T out[5];
       if (code == FV_BCK_SLIP_WALL || code == FV_BCK_NOSLIP_WALL) {
@@ -358,8 +387,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         // viscous kernel's F_v.S of this face (same face order as the
         // metrics, all blocks)
         T fva, fvb, fvc, fvd;
-        const MT* vr = reinterpret_cast<const MT*>(args.fv[dir == 0 ? 0 : (dir == 1 ? 1 : 2)]);
-        MetricStore<T>::ld4(vr, B.vface_off[dir] + (f - B.face_off[dir]), fva, fvb, fvc, fvd);
+        MetricStore<T>::ld4(s_vis[dir], f, fva, fvb, fvc, fvd);
         out[1] = out[1] - fva;
         out[2] = out[2] - fvb;
         out[3] = out[3] - fvc;
@@ -374,8 +402,22 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
     // (dir < 0: unused or outside).  Decoded on the fly: holding these in
     // registers for the whole tile costs more occupancy than the decode.
     // and (SHARE) the index of the face's lower cell in its direction's slope plane
-    auto face_item = [&](int it, int& dir, int& off, int& dst, int& hoff, long long& met) {
+    auto face_item = [&](int round, int& dir, int& off, int& dst, int& hoff, unsigned& met) {
+      const int it = tid + round * NT;
       dir = -1;
+      if constexpr (ROWS) {
+        const bool edge = tid >= 32 * TY;
+        const int y = edge ? (round == 0 ? (tid & 31) : TY) : tid >> 5, x = edge && round == 0 ? TX : (tid & 31);
+        const int i = i0 + x, j = j0 + y, ex = round == 0, ey = round == 1;
+        if (i < ni + ex && j < nj + ey && y < TY + ey) {
+          dir = round;
+          off = (y + 2 - 2 * ey) * W + (x + 2 - 2 * ex);
+          dst = y * (TX + ex) + x;
+          hoff = y * (TX + 2 * ex) + x;
+          met = (unsigned)j * (ni + ex) + i;
+        }
+        return;
+      }
       if (it < NXI) {
         // the TX faces x < TX of every row first, row by row, then the last
         // face of each row: a warp then reads whole rows of the plane
@@ -389,7 +431,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         const int i = i0 + x, j = j0 + y;
         if (i <= ni && j < nj) {
           dir = 0; off = (y + 2) * W + x; dst = y * (TX + 1) + x; hoff = y * (TX + 2) + x;
-          met = B.face_off[0] + (long long)j * (ni + 1) + i;
+          met = (unsigned)j * (ni + 1) + i;
         }
       } else if (it < NXI + NETA) {
         const int e = it - NXI;
@@ -397,14 +439,14 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         const int i = i0 + x, j = j0 + y;
         if (i < ni && j <= nj) {
           dir = 1; off = y * W + (x + 2); dst = e; hoff = e;
-          met = B.face_off[1] + (long long)j * ni + i;
+          met = (unsigned)j * ni + i;
         }
       } else if (DIM3 && it < NFACE) {
         const int e = it - NXI - NETA;
         const int y = e / TX, x = e - y * TX;
         if (i0 + x < ni && j0 + y < nj) {
           dir = 2; off = (y + 2) * W + (x + 2); dst = e; hoff = e;
-          met = B.face_off[2] + (long long)(j0 + y) * ni + (i0 + x);
+          met = (unsigned)(j0 + y) * ni + (i0 + x);
         }
       }
     };
@@ -455,7 +497,8 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         }
       }
     };
-    const long long kfx = (long long)nj * (ni + 1), kfy = (long long)(nj + 1) * ni, kfz = (long long)nj * ni;
+    // faces per plane (a block's faces of one direction stay below 2^31: their records alone would fill the memory)
+    const unsigned kfx = (unsigned)nj * (ni + 1), kfy = (unsigned)(nj + 1) * ni, kfz = (unsigned)nj * ni;
     // zeta face between planes kf-1 and kf (stencil kf-2 .. kf+1) at column offset c
     if (DIM3) {
       // planes k0-2 .. k0 now; plane k0+1 arrives in the first pass below
@@ -497,16 +540,18 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
       }
       // ---- every face of this plane (and the zeta faces above it), once;
       // one call site of the face code for all three directions ----
-      for (int it = tid; it < NFACE; it += NT) {
+      constexpr int ROUNDS = ROWS ? 2 + DIM3 : (NFACE + NT - 1) / NT;
+#pragma unroll 1
+      for (int round = ROWS && DIM3 && k < k0 ? 2 : 0; round < ROUNDS; ++round) {
         int d, off, dst, hoff;
-        long long met;
-        face_item(it, d, off, dst, hoff, met);
+        unsigned met;
+        face_item(round, d, off, dst, hoff, met);
         if (d < 0 || (DIM3 && k < k0 && d != 2)) continue;
         const T *s0, *s1, *s2, *s3, *hL, *hR;
         int hs;
         T* dp;
         int dstr;
-        long long f;
+        unsigned f;
         if (DIM3 && d == 2) {
           // zeta face between planes k and k+1: stencil k-1 .. k+2 from the ring
           // (with a 3-plane ring s0 aliases plane k+2; only the
@@ -536,25 +581,25 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
         }
         // physical boundary face with an overwritten flux?
         int code = 0, side = 0;
-        if (BC && B.bcmap) {
+        if (BC && bcmap) {
           if (d == 0) {
             const int fy = dst / (TX + 1), fi = i0 + dst - fy * (TX + 1);
             if (fi == 0 || fi == ni) {
               side = fi != 0;
-              code = B.bcmap[(side ? (long long)nj * nk : 0) + (long long)k * nj + (j0 + fy)];
+              code = bcmap[(side ? (long long)nj * nk : 0) + (long long)k * nj + (j0 + fy)];
             }
           } else if (d == 1) {
             const int fy = dst / TX, fj = j0 + fy;
             if (fj == 0 || fj == nj) {
               side = fj != 0;
-              code = B.bcmap[2LL * nj * nk + (side ? (long long)ni * nk : 0) + (long long)k * ni + (i0 + dst - fy * TX)];
+              code = bcmap[2LL * nj * nk + (side ? (long long)ni * nk : 0) + (long long)k * ni + (i0 + dst - fy * TX)];
             }
           } else {
             const int fk = k + 1;
             if (fk == 0 || fk == nk) {
               side = fk != 0;
               const int fy = dst / TX;
-              code = B.bcmap[2LL * nj * nk + 2LL * ni * nk + (side ? (long long)ni * nj : 0) +
+              code = bcmap[2LL * nj * nk + 2LL * ni * nk + (side ? (long long)ni * nj : 0) +
                              (long long)(j0 + fy) * ni + (i0 + dst - fy * TX)];
             }
           }

@@ -37,3 +37,33 @@ def test_bit_equal_to_a_given_tile(name, prec):
         s.close()
     assert np.isfinite(out[0]).all()
     assert all(np.array_equal(out[0], x) for x in out[1:])
+
+
+ROW_PROBLEMS = {
+    "below": lambda: cases.mms_3d((31, 7, 3)),
+    "exact": lambda: cases.mms_3d((32, 8, 2), curvilinear=True),
+    "above": lambda: cases.mms_3d((33, 9, 5), curvilinear=True),
+    "two": lambda: cases.mms_3d((64, 14, 4)),
+    "plane": lambda: cases.inlet_2d(104, 33, perturb=0.02, seed=1),
+    "walls": lambda: cases.ellipse_ogrid(64, 16, 7, perturb=0.02, seed=2),
+    "laminar": lambda: cases.mms_periodic_3d((33, 15, 5), curvilinear=True, visc=1, mu=0.05),
+}
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32flux"])
+@pytest.mark.parametrize("name", sorted(ROW_PROBLEMS))
+def test_row_shapes_bit_equal_to_a_listed_one(name, prec):
+    """Tiles 5 and 8 take their faces by rows of 32 cells, tile 3 from a list:
+    the same faces at the edges of tiles and blocks, bit for bit."""
+    import paper_2012_02925_gb300 as fv
+    if name == "laminar" and prec == "fp32flux":
+        pytest.skip("its temperatures are relative to each tile's first cell")
+    pb = ROW_PROBLEMS[name]()
+    out = []
+    for tile, kchunk in ((3, 2), (5, 3), (8, 2)):
+        s = fv.Solver.from_problem(pb, precision=prec, tile=tile, kchunk=kchunk)
+        s.set_state(torch.from_numpy(pb.q).cuda())
+        out.append(s.residual(0).cpu().numpy())
+        s.close()
+    assert np.isfinite(out[0]).all()
+    assert all(np.array_equal(out[0], x) for x in out[1:])
