@@ -333,9 +333,20 @@ template <> struct Sc<float> {
   static __device__ __forceinline__ float c(double x) { return (float)x; }
   // approximate (MUFU) reciprocal and square root: the binary32 flux form
   // already carries ~1e-6 relative error, a few more ulps do not matter
-  static __device__ __forceinline__ float sqrt(float x) { return x * rsqrtf(x); }
+  // (the flush-to-zero forms: without them each takes three or four more
+  // instructions to scale subnormal operands, which the face code does not
+  // have or discards; 16 of them a face)
+  static __device__ __forceinline__ float sqrt(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return x * y;
+  }
   static __device__ __forceinline__ float abs(float x) { return ::fabsf(x); }
-  static __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
+  static __device__ __forceinline__ float rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+  }
   static __device__ __forceinline__ float div(float a, float b) { return a * rcp(b); }
   static __device__ __forceinline__ float halve(float x) { return 0.5f * x; }
   static __device__ __forceinline__ float quarter(float x) { return 0.25f * x; }
