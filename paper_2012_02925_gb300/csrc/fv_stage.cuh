@@ -139,7 +139,7 @@ using StageSmemOf = StageSmem<T, TX, TY, (VISC && std::is_same<T, float>::value)
 // above the last row (eta) - so an item needs no decoding.  Same number of
 // rounds as the balanced list of the same shape.  128^3 RK step, 32 x 7 tile:
 // double-float 2.77 -> 2.46 ms, binary32 flux 0.854 -> 0.745 ms, of which the
-// block constants in shared memory (below) 4 and 9 %, as in the listed shapes.
+// block constants in shared memory (below) 6 and 9 %, as in the 32 x 8 tile.
 // (Not for the fused viscous faces, whose work hides the decoding.)
 template <int TX, int TY, int NT>
 __host__ __device__ constexpr bool stage_rows() {
@@ -203,8 +203,9 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   // The tile's block constants as the faces read them: the face records of
   // each direction (metrics, viscous fluxes), or the Cartesian unit normals
   // and areas, converted once a tile (read from the block's record at each
-  // face, with the conversions: 64-block batch in binary32 flux 4.8 against
-  // 4.4 ms, 256x256x128 periodic block in double-float 11.0 against 9.8 ms).
+  // face, with the conversions: 32-block batch in binary32 flux, 16 x 8 tile,
+  // 2.41 against 2.17 ms; 256x256x128 periodic block in double-float, 32 x 8
+  // tile, 11.0 against 9.8 ms).
   __shared__ const MT* s_met[3];
   __shared__ const MT* s_vis[3];
   __shared__ __align__(16) T s_cart[12];
