@@ -47,11 +47,10 @@ template <> struct AdjMem<df64> {
 // cell sweep each read a cell's primitives up to twelve times.  (Corner
 // ghosts hold no data; nothing reads theirs.)
 template <class T>
-__global__ void adj_prim_kernel(const FvBlockDev B, const double* __restrict__ qin, const AdjParams PP,
+__global__ void adj_prim_kernel(const FvBlockDev B, const double* __restrict__ qin, const AdjC<T> P,
                                 typename AdjMem<T>::type* __restrict__ prim) {
   using S = Sc<T>;
   using M = AdjMem<T>;
-  const AdjC<T> P = adj_consts<T>(PP);
   for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < B.plane;
        x += (long long)gridDim.x * blockDim.x) {
     T q[5];
@@ -78,11 +77,10 @@ __global__ void __launch_bounds__(NT, MINB) adj_face_kernel(const FvBlockDev B, 
                                                        const typename AdjMem<T>::type* __restrict__ prim,
                                                        const double* __restrict__ lam_out,
                                                        const double* __restrict__ invvol, double alpha_dt,
-                                                       const double* __restrict__ metric, const AdjParams PP,
+                                                       const double* __restrict__ metric, const AdjC<T> P,
                                                        typename AdjMem<T>::type* __restrict__ out) {
   using S = Sc<T>;
   using M = AdjMem<T>;
-  const AdjC<T> P = adj_consts<T>(PP);
   const int ei = B.ni + (dir == 0), ej = B.nj + (dir == 1), ek = B.nk + (dir == 2);
   const long long nf = (long long)ei * ej * ek;
   const long long ncell_b = (long long)B.ni * B.nj * B.nk;
@@ -159,10 +157,9 @@ template <class T>
 __global__ void __launch_bounds__(128) adj_slope_kernel(const FvBlockDev B, int dir,
                                                         const typename AdjMem<T>::type* __restrict__ prim,
                                                         const typename AdjMem<T>::type* __restrict__ cot,
-                                                        const AdjParams PP, typename AdjMem<T>::type* __restrict__ out) {
+                                                        const AdjC<T> P, typename AdjMem<T>::type* __restrict__ out) {
   using S = Sc<T>;
   using M = AdjMem<T>;
-  const AdjC<T> P = adj_consts<T>(PP);
   const int ei = B.ni + (dir == 0), ej = B.nj + (dir == 1), ek = B.nk + (dir == 2);
   const int ci = B.ni + 2 * (dir == 0), cj = B.nj + 2 * (dir == 1), ck = B.nk + 2 * (dir == 2);
   const long long nf = (long long)ei * ej * ek, nc = (long long)ci * cj * ck;
@@ -205,12 +202,11 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const
                                                        const typename AdjMem<T>::type* __restrict__ sx,
                                                        const typename AdjMem<T>::type* __restrict__ sy,
                                                        const typename AdjMem<T>::type* __restrict__ sz, int three_d,
-                                                       const AdjParams PP, double* __restrict__ lamg,
+                                                       const AdjC<T> P, double* __restrict__ lamg,
                                                        const double* __restrict__ lam_out, double* __restrict__ lam_in,
                                                        double* __restrict__ lam_q0) {
   using S = Sc<T>;
   using M = AdjMem<T>;
-  const AdjC<T> P = adj_consts<T>(PP);
   const int g = lam_in ? 0 : FV_GHOST;
   const int gi = B.ni + 2 * g, gj = B.nj + 2 * g, gk = B.nk + 2 * g;
   const long long n = (long long)gi * gj * gk;
@@ -337,7 +333,7 @@ int adjoint_block(const FvBlockDev& B, int nd, const double* qin, const double* 
                   double alpha_dt, const double* const metric[3], const FvFaceParams& fp, void* prim_mem, void* cot_mem,
                   void* slope_mem, double* lamg, double* lam_in, double* lam_q0, cudaStream_t s) {
   using MT = typename AdjMem<T>::type;
-  const AdjParams P = adj_params(fp);
+  const AdjC<T> P = adj_consts<T>(adj_params(fp));
   MT* prim = static_cast<MT*>(prim_mem);
   MT* cot = static_cast<MT*>(cot_mem);
   adj_prim_kernel<T><<<grid_of(B.plane, 256), 256, 0, s>>>(B, qin, P, prim);

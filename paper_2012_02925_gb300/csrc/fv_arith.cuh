@@ -72,7 +72,7 @@ struct df64 {
   float hi, lo;
 };
 
-FV_HD df64 mk(float h, float l) { df64 r; r.hi = h; r.lo = l; return r; }
+__host__ __device__ __forceinline__ df64 mk(float h, float l) { df64 r; r.hi = h; r.lo = l; return r; }
 
 // binary32 operations that the compiler may neither contract into FMAs nor
 // reorder: the error-free transformations below depend on every rounding.
@@ -274,7 +274,7 @@ template <class T> struct Sc;
 template <> struct Sc<double> {
   static __device__ __forceinline__ double from_d(double x) { return x; }
   static __device__ __forceinline__ double to_d(double x) { return x; }
-  static __device__ __forceinline__ double c(double x) { return x; }     // constant
+  static __host__ __device__ __forceinline__ double c(double x) { return x; }     // constant
   static __device__ __forceinline__ double sqrt(double x) { return fv_sqrt64(x); }
   static __device__ __forceinline__ double abs(double x) { return ::fabs(x); }
   // reciprocal within one unit in the last place (fv_rcp64); a quotient is
@@ -330,7 +330,7 @@ template <> struct Sc<float> {
   // zero rather than to nearest: 4 % faster again, within the form's error
   static __device__ __forceinline__ float from_d(double x) { return fv_d2f_rz(x); }
   static __device__ __forceinline__ double to_d(float x) { return fv_f2d(x); }
-  static __device__ __forceinline__ float c(double x) { return (float)x; }
+  static __host__ __device__ __forceinline__ float c(double x) { return (float)x; }
   // approximate (MUFU) reciprocal and square root: the binary32 flux form
   // already carries ~1e-6 relative error, a few more ulps do not matter
   // (the flush-to-zero forms: without them each takes three or four more
@@ -380,8 +380,8 @@ template <> struct Sc<float> {
 template <> struct Sc<df64> {
   static __device__ __forceinline__ df64 from_d(double x) { return fv_d2df(x); }
   static __device__ __forceinline__ double to_d(df64 x) { return fv_df2d(x); }
-  // compile-time constants: split on the host side of the compiler
-  static __device__ __forceinline__ df64 c(double x) {
+  // constants: split by the compiler, or on the host before a launch
+  static __host__ __device__ __forceinline__ df64 c(double x) {
     float h = (float)x;
     return mk(h, (float)(x - (double)h));
   }

@@ -67,10 +67,16 @@ template <> struct Acc<float> {
   static __device__ __forceinline__ df64 from_d(double x) { return fv_d2df(x); }
 };
 
+// binary64 factors of the update in the form's arithmetic
+template <class T> struct Upd {
+  static __device__ __forceinline__ T from_d(double x) { return Sc<T>::from_d(x); }
+};
+template <> struct Upd<float> {
+  static __device__ __forceinline__ float from_d(double x) { return fv_d2f_rn(x); }
+};
+
 // Q^(0) - fac * R in binary64, with fac = alpha dt / Omega
-__device__ __forceinline__ double rk_apply(double q0, double alpha_dt, double invvol, double R) {
-  return q0 - (alpha_dt * invvol) * R;
-}
+__device__ __forceinline__ double rk_apply(double q0, double fac, double R) { return q0 - fac * R; }
 __device__ __forceinline__ double rk_apply(double q0, df64 fac, df64 R) {
   df64 d = fac * R;
   return q0 - fv_df2d(d);
@@ -153,6 +159,20 @@ constexpr int stage_min_ctas() {
   return sizeof(T) == 4 ? (VISC ? (NT <= 128 ? 6 : 3) : (NT <= 128 ? 8 : 4)) : (NT <= 128 ? 4 : (NT <= 256 ? 2 : 1));
 }
 
+// a launch's constants in the arithmetic type (host)
+template <class T>
+struct StageC {
+  FaceC<T> face;
+  ViscC<T> visc;
+  df64 gm1;      // gamma - 1 and 1 / R of the fused viscous terms
+  float iR;
+};
+template <class T>
+inline StageC<T> make_stage_consts(const FvStageArgs& a) {
+  return StageC<T>{make_face_consts<T>(a.fp), make_visc_consts<T>(a.vp), Sc<df64>::c(a.vp.gamma - 1.0),
+                   (float)(1.0 / a.vp.r_gas)};
+}
+
 // VISC: the laminar viscous terms.  The binary32 form evaluates them in the
 // face loop (FUSED_VISC); the wider forms subtract the per-face fluxes of the
 // separate viscous kernel from each face's inviscid flux in the face loop
@@ -163,7 +183,8 @@ constexpr int stage_min_ctas() {
 // face) their code is not compiled in, which on the 128^3 block made both
 // the double-float and the binary32 kernels 10 % faster.
 template <class T, int TX, int TY, int NT, bool DIM3, bool PF, bool FAST, bool VISC, bool BC>
-__global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_kernel(const FvStageArgs args) {
+__global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_kernel(const FvStageArgs args,
+                                                                                   const StageC<T> consts) {
   constexpr bool FUSED_VISC = VISC && std::is_same<T, float>::value;
   constexpr bool VISC_PAIRS = VISC && !std::is_same<T, float>::value;
   using S = Sc<T>;
@@ -197,8 +218,8 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   };
 
   const int tid = threadIdx.x;
-  const CC C = CC::from(make_face_consts<T>(args.fp));
-  const ViscC<T> VK = make_visc_consts<T>(args.vp);
+  const CC C = CC::from(consts.face);
+  const ViscC<T>& VK = consts.visc;
   const typename VGeo<T>::type* geo = reinterpret_cast<const typename VGeo<T>::type*>(args.geo);
   // The tile's block constants as the faces read them: the face records of
   // each direction (metrics, viscous fluxes), or the Cartesian unit normals
@@ -209,6 +230,11 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   __shared__ const MT* s_met[3];
   __shared__ const MT* s_vis[3];
   __shared__ __align__(16) T s_cart[12];
+  // alpha_m dt (the binary64 product the host forms when dt is passed by
+  // value), and times a Cartesian block's 1/Omega, in the update's arithmetic
+  __shared__ T s_fac;
+  const double alpha_dt = args.dt_dev ? args.alpha * *args.dt_dev : args.alpha_dt;
+  const T adt = Upd<T>::from_d(alpha_dt);
 
   // Tiles 0..gridDim-1 go to the CTAs in order; later ones are handed out
   // dynamically (largest first, as the table is sorted) through a counter
@@ -229,6 +255,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
       s_met[tid] = reinterpret_cast<const MT*>(args.metric[tid]) + 4 * B.face_off[tid];
       if (VISC_PAIRS) s_vis[tid] = reinterpret_cast<const MT*>(args.fv[tid]) + 4 * B.vface_off[tid];
     }
+    if (cart && tid == 0) s_fac = adt * Upd<T>::from_d(B.cart_invvol);
     if (cart && tid < 12) {
       const int d = tid >> 2, x = tid & 3;
       s_cart[tid] = S::from_d(x < 3 ? B.cart_n[d][x] : B.cart_area[d]);
@@ -262,8 +289,8 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
                      (r * r * args.vp.r_gas));
       trefR = fv_d2df((double)tref * args.vp.r_gas);
     }
-    const df64 gm1_df = Sc<df64>::c(args.vp.gamma - 1.0);
-    const float iR_f = (float)(1.0 / args.vp.r_gas);
+    const df64 gm1_df = consts.gm1;
+    const float iR_f = consts.iR;
     auto t_dev = [&](const double* qd, float rho) -> float {
       const df64 r = fv_d2df(qd[0]), m1 = fv_d2df(qd[1]), m2 = fv_d2df(qd[2]), m3 = fv_d2df(qd[3]);
       const df64 e = fv_d2df(qd[4]);
@@ -696,22 +723,18 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
             }
           }
           if (args.mode == FV_MODE_RK) {
-            // the same binary64 product the host forms when dt is passed by value
-            const double alpha_dt = args.dt_dev ? args.alpha * *args.dt_dev : args.alpha_dt;
-            const double iv = cart ? B.cart_invvol : __ldg(args.invvol + B.cell_off + cell);
+            const T fac = cart ? s_fac : adt * Upd<T>::from_d(__ldg(args.invvol + B.cell_off + cell));
             const double* q0 = args.q0 + B.qoff + q_idx;
             double* qo = args.qout + B.qoff + q_idx;
             if constexpr (std::is_same<AT, double>::value) {
 #pragma unroll
-              for (int n = 0; n < 5; ++n) qo[n * pl] = rk_apply(q0[n * pl], alpha_dt, iv, R[n]);
+              for (int n = 0; n < 5; ++n) qo[n * pl] = rk_apply(q0[n * pl], fac, R[n]);
             } else if constexpr (std::is_same<T, float>::value) {
               // binary32 increment (its rounding is far below the error of
               // the binary32 face fluxes it sums), one binary64 add
-              const float fac = FMUL(fv_d2f_rn(alpha_dt), fv_d2f_rn(iv));
 #pragma unroll
               for (int n = 0; n < 5; ++n) qo[n * pl] = q0[n * pl] - fv_f2d(FMUL(fac, FADD(R[n].hi, R[n].lo)));
             } else {
-              const df64 fac = fv_d2df(alpha_dt) * fv_d2df(iv);
 #pragma unroll
               for (int n = 0; n < 5; ++n) qo[n * pl] = rk_apply(q0[n * pl], fac, R[n]);
             }
@@ -762,10 +785,11 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
 template <class T, int TX, int TY, int NT, bool PF, bool FAST, bool VISC, bool BC>
 static int launch_stage_t(const FvStageArgs& a, const FvLaunch& l, cudaStream_t s) {
   const size_t smem = StageSmemOf<T, TX, TY, FAST, VISC, BC>::bytes(l.three_d != 0, PF);
+  const StageC<T> c = make_stage_consts<T>(a);
   if (l.three_d) {
-    fv_stage_kernel<T, TX, TY, NT, true, PF, FAST, VISC, BC><<<l.grid, NT, smem, s>>>(a);
+    fv_stage_kernel<T, TX, TY, NT, true, PF, FAST, VISC, BC><<<l.grid, NT, smem, s>>>(a, c);
   } else {
-    fv_stage_kernel<T, TX, TY, NT, false, false, FAST, VISC, BC><<<l.grid, NT, smem, s>>>(a);
+    fv_stage_kernel<T, TX, TY, NT, false, false, FAST, VISC, BC><<<l.grid, NT, smem, s>>>(a, c);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

@@ -59,7 +59,7 @@ struct ViscC {
   int sutherland;
 };
 template <class T>
-__device__ __forceinline__ ViscC<T> make_visc_consts(const FvViscParams& p) {
+inline ViscC<T> make_visc_consts(const FvViscParams& p) {
   using S = Sc<T>;
   ViscC<T> v;
   v.iR = S::c(1.0 / p.r_gas);
