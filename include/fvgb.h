@@ -171,7 +171,8 @@ typedef struct {
  *     5: 32x8 / 288, 6: 32x8 / 256 and 7: 32x4 / 128 with the next k-plane
  *     prefetched by cp.async - 6 and 7 for FV_PREC_FP32FLUX only -, 8: 32x7 / 256,
  *     9: 32x6 / 256, 10: 16x12 / 192, 11: 16x4 / 128, 12: 8x8 / 128 -
- *     FV_PREC_FP64 only).
+ *     FV_PREC_FP64 only -, 13: 8x8 / 160 - 2-D only; 11 in the place of a
+ *     number beyond these or of 12 and 13 where they do not exist).
  *   kchunk: k-planes per tile; 0 = automatic (about three tiles per resident
  *     CTA slot when the tile shape is given); -w = about w tiles per resident CTA slot.  Tiles are handed
  *     to persistent CTAs largest first through a device counter.

@@ -861,9 +861,15 @@ int copy_state(fv_ctx* h, const double* src, double* dst, bool to_internal, cuda
   return FV_OK;
 }
 
+// the shape a given tile number stands for: 16 x 4 for numbers beyond the
+// table and for the shapes that the form or dimension does not have
+int given_shape(const fv_config& c) {
+  if (c.tile > FV_NUM_SHAPES || (c.tile == 12 && c.precision != FV_PREC_FP64) || (c.tile == 13 && c.dim == 3)) return 11;
+  return c.tile;
+}
+
 void set_shape(fv_ctx* h, int shape) {
   FvLaunch& l = h->launch;
-  shape = std::min(std::max(shape, 1), FV_NUM_SHAPES);
   l.shape = shape;
   l.tx = FV_SHAPE_TABLE[shape - 1][0];
   l.ty = FV_SHAPE_TABLE[shape - 1][1];
@@ -919,7 +925,9 @@ int kchunk_of(const FvBlockDev& b, int dim, int kchunk, long long slots, long lo
 // 10.9 M cells, RK step with the fixed 32 x 8 shape (16 x 8 for narrow blocks)
 // over this rule's: binary64 1.2 .. 2.5, double-float 1.0 .. 2.2,
 // binary32 flux 1.0 .. 2.0; 64-block batch in binary64 39.3 -> 24.7 ms, in
-// binary32 flux 5.23 -> 4.74 ms.
+// binary32 flux 5.23 -> 4.74 ms.  (8 x 8 with 160 threads, 2-D: its cost makes
+// it the choice while every tile has a slot at once; 64^2 vortex 70 -> 58 us,
+// at 192^2 it would take 105 us where the rule's pick takes 93.)
 void choose_launch(fv_ctx* h) {
   const fv_config& c = h->cfg;
   FvLaunch l{};
@@ -935,17 +943,17 @@ void choose_launch(fv_ctx* h) {
   h->launch = l;
   h->kchunk = c.kchunk;
   if (c.tile > 0) {
-    set_shape(h, c.tile);
+    set_shape(h, given_shape(c));
     return;
   }
   struct Shape { int id, ref; double cost; };
-  static const Shape tables[2][3][6] = {
+  static const Shape tables[2][3][8] = {
       {{{12, 4, 4.35}, {11, 4, 4.42}, {9, 2, 4.33}, {3, 3, 4.51}},                                 // 3-D: binary64
-       {{1, 2, 2.73}, {8, 2, 2.75}, {9, 2, 2.97}, {11, 4, 3.87}},                                  // double-float
-       {{1, 4, 0.92}, {8, 4, 0.93}, {9, 4, 0.96}, {3, 7, 0.97}, {11, 8, 1.08}}},                   // binary32 flux
-      {{{11, 4, 5.75}, {9, 2, 5.26}, {3, 4, 4.67}, {8, 2, 4.81}},                                  // 2-D
-       {{1, 2, 3.56}, {8, 2, 3.38}, {9, 2, 3.76}, {3, 4, 3.64}, {11, 4, 4.40}},
-       {{1, 4, 1.29}, {8, 4, 1.27}, {9, 4, 1.35}, {3, 8, 1.28}, {11, 8, 1.51}}}};
+       {{1, 2, 2.47}, {8, 2, 2.39}, {9, 2, 2.74}, {11, 4, 3.53}},                                  // double-float
+       {{1, 4, 0.80}, {8, 4, 0.68}, {5, 4, 0.73}, {9, 4, 0.89}, {3, 7, 0.80}, {11, 8, 0.92}}},                   // binary32 flux
+      {{{13, 2, 9.90}, {11, 4, 5.75}, {9, 2, 5.26}, {3, 4, 4.67}, {8, 2, 4.81}},                                  // 2-D
+       {{13, 2, 7.60}, {1, 2, 3.56}, {8, 2, 3.38}, {9, 2, 3.76}, {3, 4, 3.64}, {11, 4, 4.40}},
+       {{13, 4, 2.70}, {1, 4, 1.29}, {8, 4, 1.27}, {9, 4, 1.35}, {3, 8, 1.28}, {11, 8, 1.51}}}};
   const int form = c.precision == FV_PREC_FP64 ? 0 : (c.precision == FV_PREC_DF64 ? 1 : 2);
   const Shape* table = tables[c.dim == 2][form];
   static const int chunks[] = {0, -1, -2, 4, 8, 16, 32};
@@ -1850,6 +1858,7 @@ int fv_autotune(fv_handle hh, double dt, int reps, void* stream) {
       if (h->cfg.dim == 2 && kc != 0) continue;
       h->cfg.tile = tile;
       h->cfg.kchunk = kc;
+      if (given_shape(h->cfg) != tile) continue;
       choose_launch(h);
       if (build_tiles(h) != FV_OK) continue;
       int rc = do_stage(h, 1, dt, s);

@@ -782,26 +782,29 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
 
 // The dynamic shared-memory limit is raised once by occupancy_t (at handle
 // creation), so a launch is a plain enqueue that stream capture accepts.
-template <class T, int TX, int TY, int NT, bool PF, bool FAST, bool VISC, bool BC>
+template <class T, int TX, int TY, int NT, bool PF, bool FAST, bool VISC, bool BC, bool PLANE>
 static int launch_stage_t(const FvStageArgs& a, const FvLaunch& l, cudaStream_t s) {
   const size_t smem = StageSmemOf<T, TX, TY, FAST, VISC, BC>::bytes(l.three_d != 0, PF);
   const StageC<T> c = make_stage_consts<T>(a);
   if (l.three_d) {
-    fv_stage_kernel<T, TX, TY, NT, true, PF, FAST, VISC, BC><<<l.grid, NT, smem, s>>>(a, c);
+    if constexpr (PLANE) return -2;
+    else fv_stage_kernel<T, TX, TY, NT, true, PF, FAST, VISC, BC><<<l.grid, NT, smem, s>>>(a, c);
   } else {
     fv_stage_kernel<T, TX, TY, NT, false, false, FAST, VISC, BC><<<l.grid, NT, smem, s>>>(a, c);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-template <class T, int TX, int TY, int NT, bool PF, bool FAST, bool VISC, bool BC>
+template <class T, int TX, int TY, int NT, bool PF, bool FAST, bool VISC, bool BC, bool PLANE>
 static int occupancy_t(bool three_d, size_t* smem_out) {
   const size_t smem = StageSmemOf<T, TX, TY, FAST, VISC, BC>::bytes(three_d, PF);
   int n = 0;
   if (three_d) {
-    auto k = fv_stage_kernel<T, TX, TY, NT, true, PF, FAST, VISC, BC>;
-    cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, NT, smem);
+    if constexpr (!PLANE) {
+      auto k = fv_stage_kernel<T, TX, TY, NT, true, PF, FAST, VISC, BC>;
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, NT, smem);
+    }
   } else {
     auto k = fv_stage_kernel<T, TX, TY, NT, false, false, FAST, VISC, BC>;
     cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -817,7 +820,11 @@ static int occupancy_t(bool three_d, size_t* smem_out) {
 // the wider forms a resident CTA), the square 64-cell one for binary64 only
 // (fewer halo cells, faces and slopes than 16 x 4: 64-block batch 25.3 -> 24.0
 // ms, 128^3 4.42 -> 4.35 ms in that shape; its rows of 64 bytes do not matter
-// to a kernel at 6 % of the memory bandwidth).
+// to a kernel at 6 % of the memory bandwidth).  8 x 8 with 160 threads is for
+// small 2-D problems, whose time is the length of one tile's chain: its 144
+// staged cells, 160 slopes and 144 faces are one round each (64^2 vortex
+// RK step: binary64 70 -> 58 us, double-float 54 -> 47; 104 x 32 inlet: 78 -> 62,
+// 64 -> 54, binary32 flux 47 -> 43).
 #define FV_SHAPES(X)      \
   X(1, 32, 8, 256, false) \
   X(2, 32, 4, 128, false) \
@@ -830,7 +837,8 @@ static int occupancy_t(bool three_d, size_t* smem_out) {
   X(9, 32, 6, 256, false) \
   X(10, 16, 12, 192, false) \
   X(11, 16, 4, 128, false) \
-  X(12, 8, 8, 128, false)
+  X(12, 8, 8, 128, false) \
+  X(13, 8, 8, 160, false)
 
 // FAST selects the compile-time default scheme (FaceCFast); each
 // translation unit instantiates one combination of FAST, VISC and BC.
@@ -840,7 +848,7 @@ int fv_dispatch_launch(const FvStageArgs& a, const FvLaunch& l, cudaStream_t s) 
 #define FV_LAUNCH_CASE(ID, TX, TY, NT, PF)                                     \
   if (l.shape == ID) {                                                          \
     if ((PF && !allow_pf) || (ID == 12 && !wide)) return -2;                    \
-    return launch_stage_t<T, ID == 12 && !wide ? 16 : TX, ID == 12 && !wide ? 4 : TY, NT, PF && allow_pf, FAST, VISC, BC>(a, l, s); \
+    return launch_stage_t<T, ID == 12 && !wide ? 16 : TX, ID == 12 && !wide ? 4 : TY, NT, PF && allow_pf, FAST, VISC, BC, ID == 13>(a, l, s); \
   }
   FV_SHAPES(FV_LAUNCH_CASE)
 #undef FV_LAUNCH_CASE
@@ -854,7 +862,7 @@ int fv_dispatch_occupancy(const FvLaunch& l, size_t* smem) {
 #define FV_OCC_CASE(ID, TX, TY, NT, PF)                                         \
   if (l.shape == ID) {                                                          \
     if ((PF && !allow_pf) || (ID == 12 && !wide)) return 0;                     \
-    return occupancy_t<T, ID == 12 && !wide ? 16 : TX, ID == 12 && !wide ? 4 : TY, NT, PF && allow_pf, FAST, VISC, BC>(d3, smem); \
+    return occupancy_t<T, ID == 12 && !wide ? 16 : TX, ID == 12 && !wide ? 4 : TY, NT, PF && allow_pf, FAST, VISC, BC, ID == 13>(d3, smem); \
   }
   FV_SHAPES(FV_OCC_CASE)
 #undef FV_OCC_CASE

@@ -67,3 +67,20 @@ def test_row_shapes_bit_equal_to_a_listed_one(name, prec):
         s.close()
     assert np.isfinite(out[0]).all()
     assert all(np.array_equal(out[0], x) for x in out[1:])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32flux"])
+@pytest.mark.parametrize("name", ["vortex", "inlet", "narrow"])
+def test_tile_numbers_without_a_shape(name, prec):
+    """12 exists in binary64 only, 13 in 2-D only; these and larger numbers
+    run everywhere, bit-equal to 11."""
+    import paper_2012_02925_gb300 as fv
+    pb = PROBLEMS[name]()
+    out = []
+    for tile in (11, 12, 13, 99):
+        s = fv.Solver.from_problem(pb, precision=prec, tile=tile)
+        s.set_state(torch.from_numpy(pb.q).cuda())
+        out.append(s.residual(0).cpu().numpy())
+        s.close()
+    assert np.isfinite(out[0]).all()
+    assert all(np.array_equal(out[0], x) for x in out[1:])
