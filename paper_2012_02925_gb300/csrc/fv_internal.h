@@ -43,10 +43,14 @@ struct FvConnDev {
   long long item_off;           // first work item (a, b, depth) of this connection
 };
 
-// One unit of work of the exchange kernel: items a0..a0+FV_XCH_TA-1 x
-// b0..b0+FV_XCH_TB-1 (both depths) of connection `conn`, clipped to its patch.
+// One unit of work of the exchange kernel: na x nb positions (a, b) of a
+// connection and both depths d = 0, 1, copied from src + a sa + b sb + d sd to
+// dst + a da + b db + d dd, the variables splane and dplane apart.  fs, fd: the
+// index (0 a, 1 b, 2 depth) that runs along the memory of each side.
 struct FvXchTile {
-  int conn, a0, b0, pad_;
+  int na, nb, fs, fd;
+  long long src, sa, sb, sd, splane;
+  long long dst, da, db, dd, dplane;
 };
 constexpr int FV_XCH_TA = 32, FV_XCH_TB = 16;
 
