@@ -942,10 +942,10 @@ void choose_launch(fv_ctx* h) {
     return;
   }
   struct Shape { int id, ref; double cost; };
-  static const Shape tables[2][3][8] = {
+  static const Shape tables[2][3][7] = {
       {{{12, 4, 4.35}, {11, 4, 4.42}, {9, 2, 4.33}, {3, 3, 4.51}},                                 // 3-D: binary64
-       {{1, 2, 2.47}, {8, 2, 2.39}, {9, 2, 2.74}, {11, 4, 3.53}},                                  // double-float
-       {{1, 4, 0.80}, {8, 4, 0.68}, {5, 4, 0.73}, {9, 4, 0.89}, {3, 7, 0.80}, {11, 8, 0.92}}},                   // binary32 flux
+       {{1, 2, 2.73}, {8, 2, 2.75}, {9, 2, 2.97}, {11, 4, 3.87}},                                  // double-float
+       {{1, 4, 0.92}, {8, 4, 0.93}, {9, 4, 0.96}, {3, 7, 0.97}, {11, 8, 1.08}}},                   // binary32 flux
       {{{13, 2, 9.90}, {11, 4, 5.75}, {9, 2, 5.26}, {3, 4, 4.67}, {8, 2, 4.81}},                                  // 2-D
        {{13, 2, 7.60}, {1, 2, 3.56}, {8, 2, 3.38}, {9, 2, 3.76}, {3, 4, 3.64}, {11, 4, 4.40}},
        {{13, 4, 2.70}, {1, 4, 1.29}, {8, 4, 1.27}, {9, 4, 1.35}, {3, 8, 1.28}, {11, 8, 1.51}}}};
