@@ -70,12 +70,14 @@ def alu_ops_per_cell(dim: int = 3, visc: bool = False) -> int:
 def alu_peak(precision: str, rates: dict):
     """Measured FP64-operation roofline of the arithmetic forms and how it
     was obtained.  binary64: twice the measured binary64 FMA rate (FLOP/s,
-    an FMA counted as two operations).  double-float: the measured rate of
+    an FMA counted as two operations), although that form's Roe flux and
+    limiter run on the integer units.  double-float: the measured rate of
     the face's operation mix, sum_k n_k / sum_k (n_k / rate_k) over the
     oracle's per-face counts n_k of add, multiply, divide, square root and
     absolute value and the measured double-float rate of each."""
     if precision == "fp64":
-        return 2.0 * rates["fp64_fma"], "measured: 2 x binary64 FMA rate (fv_probe_alu_rates)"
+        return 2.0 * rates["fp64_fma"], ("measured: 2 x binary64 FMA rate (fv_probe_alu_rates); the Roe flux and the limiter run on "
+                                         "the integer units, so the fraction can exceed 1")
     key = {"add": "df64_add", "mul": "df64_mul", "div": "df64_div", "sqrt": "df64_sqrt", "abs": "df64_abs"}
     t = sum(FACE_OPS[k] / rates[key[k]] for k in FACE_OPS)
     return sum(FACE_OPS.values()) / t, "measured: double-float rates over the face's operation mix"
