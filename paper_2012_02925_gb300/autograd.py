@@ -16,7 +16,7 @@ states.
 
 Everything numerical runs in the library's kernels; this module copies
 states in and out of the library's buffers and maps between the packed
-ghosted layout and the packed interior field (strided copies or index gathers).
+ghosted layout and the packed interior field (index gathers).
 """
 from __future__ import annotations
 
@@ -44,38 +44,13 @@ def _interior_index(solver) -> torch.Tensor:
     return idx
 
 
-# Up to this many blocks the interior is copied block by block through strided
-# views; with more, one gather or scatter by an index table is fewer launches.
-# One 96^3 block, four stages and their gradient: 6.29 ms with the table, 6.16
-# with the views, and no table to build and upload at the first pass (1.2 ms).
-_VIEW_BLOCKS = 8
-
-
-def _interior_views(solver, q: torch.Tensor):
-    """Each block's interior cells in the packed ghosted state, (5, nk, nj, ni)."""
-    off = 0
-    for ni, nj, nk in solver.block_dims:
-        n = 5 * (ni + 4) * (nj + 4) * (nk + 4)
-        yield q[off:off + n].view(5, nk + 4, nj + 4, ni + 4)[:, 2:-2, 2:-2, 2:-2]
-        off += n
-
-
 def interior(solver, q: torch.Tensor) -> torch.Tensor:
-    if len(solver.block_dims) > _VIEW_BLOCKS:
-        return q.index_select(0, _interior_index(solver))
-    parts = [v.reshape(-1) for v in _interior_views(solver, q.contiguous())]
-    return parts[0] if len(parts) == 1 else torch.cat(parts)
+    return q.index_select(0, _interior_index(solver))
 
 
 def scatter_interior(solver, field: torch.Tensor) -> torch.Tensor:
     out = torch.zeros(solver.state_size, dtype=torch.float64, device=field.device)
-    if len(solver.block_dims) > _VIEW_BLOCKS:
-        out.index_copy_(0, _interior_index(solver), field)
-        return out
-    off = 0
-    for v in _interior_views(solver, out):
-        v.copy_(field[off:off + v.numel()].view(v.shape))
-        off += v.numel()
+    out.index_copy_(0, _interior_index(solver), field)
     return out
 
 
