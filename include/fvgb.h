@@ -66,7 +66,8 @@ typedef enum {
 typedef enum {
   FV_PREC_FP64 = 0,      /* IEEE binary64; the Roe flux of a face in 64-bit
                             fixed point with the face's own scales where the
-                            face fits them (error below binary64's) */
+                            face fits them (error of each component no larger
+                            than binary64's, at any Mach number) */
   FV_PREC_DF64 = 1,      /* face arithmetic in double-float (pairs of binary32,
                             ~48-bit significand) on the FP32 pipe */
   FV_PREC_FP32FLUX = 2   /* limiter / reconstruction / Roe flux in binary32;

@@ -4,16 +4,28 @@
 // GB300's FP64 unit issues 1.6 lanes per SM and clock, so one binary64
 // operation occupies 80 of an SM's 128-lane issue slots; a signed 64 x 64 ->
 // high 64 bit product costs about 23 (two IMAD.HI at 4.5, a signed wide IMAD
-// at 9, the carries) and a 64-bit sum 3 (measured on the part).  Every quantity of the face is held with an absolute
-// resolution of 2^-60 .. 2^-71 of the face's scales, so that a flux carries
-// 2^-55 .. 2^-57 of its terms, where binary64 rounds each of its ~126
-// operations to 2^-53.
+// at 9, the carries) and a 64-bit sum 3 (measured on the part).
+//
+// Two scales a face: the thermodynamic quantities and the speed (rho, p, c~,
+// h, |u|^2) on the larger, what is proportional to the normal velocity or to
+// the jumps (Vn, the mass flux, wave strengths, the energy flux) on one of
+// their own, 2^-kn of it.  Both leave 2^-55 .. 2^-57 of the largest term of each
+// quantity, where binary64 rounds each of its ~126 operations to 2^-53.  Vn
+// and the momentum flux are binary64 (20 operations: a velocity component or a
+// normal's may be any amount smaller than the others, and its momentum flux
+// follows it).  So every component of the flux is as accurate as binary64's,
+// at any Mach number: root mean squares of the error 0.4 .. 1.05 of its
+// (tests/test_fixed_roe_accuracy.py).  With one scale and an integer momentum
+// flux the 128^3 RK step took 4.20 ms instead of 4.68, but the mass flux had an error of
+// 2^-64 of the speed of sound's, 100 times binary64's at Mach 0.001, and a
+// momentum component lost the digits by which its velocity was the smaller.
 //
 // Scales: rho^ = rho 2^-mr in [1/4, 1/2) for the denser side, velocities
 // u^ = u 2^-mv with |u^|^2 + 2 gamma/(gamma-1) p^/rho^ < 0.026 on both sides,
-// p^ = p 2^-(mr + 2 mv).  They depend on the face's two states only, so a face
-// has the same flux in whatever tile or block it is evaluated.  Formats
-// ("Qn": integer = value 2^n): rho, velocities Q64; p Q71; normals Q62.
+// p^ = p 2^-(mr + 2 mv), Vn^ = Vn 2^-mv < 2^-4-kn or kn = 0.  They depend on the
+// face's two states and normal only, so a face has the same flux in whatever
+// tile or block it is evaluated.  Formats
+// ("Qn": integer = value 2^n): rho, velocities Q64; p Q71; Vn Q(64 + kn).
 // Ranges that follow from the scales are stated at each line; what they do
 // not confine (wave strengths, the flux) is checked, and a face outside its
 // ranges (density ratio above about 4, sound speed ratio or Mach number too large,
@@ -64,11 +76,14 @@ FX_HD fx64 fx_mul(fx64 a, fx64 b) {
   const int cross = fx_madhi(ah, bl, fx_madhi(al, bh, 0));
   return fx_prod(ah, bh) + cross;
 }
-FX_HD fx64 fx_sqr(fx64 a) {
-  int ah, al;
-  fx_split(a, ah, al);
-  const int cross = fx_madhi(ah, al, 0);
-  return fx_prod(ah, ah) + 2 * (fx64)cross;
+// a^2 / 2^64 of a magnitude below 2^63 (a number and its negative thus have the same square)
+FX_HD fx64 fx_usqr(fxu64 a) {
+  const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+  return (fx64)((fxu64)ah * ah + fx_umulhi(2 * ah, al));
+}
+FX_HD fxu64 fx_abs(fx64 a) {
+  const fx64 s = a >> 63;
+  return (fxu64)((a ^ s) - s);
 }
 // a b / 2^64 of non-negative numbers below 2^63
 FX_HD fx64 fx_umul(fx64 a, fx64 b) {
@@ -76,21 +91,11 @@ FX_HD fx64 fx_umul(fx64 a, fx64 b) {
   fxu64 t = (fxu64)al * bh + 0x80000000u;
   t = (fxu64)ah * bl + t;
   return (fx64)((fxu64)ah * bh + (t >> 32));
-}
-// (a . b) / 2^64 of three-vectors, |a| Q62 unit vector, |b_i| < 2^63 0.4 (the
-// six cross products then sum within 32 bits)
-FX_HD fx64 fx_dot3(const fx64 a[3], const fx64 b[3]) {
-  int cross = 0;
-  fx64 s = 0;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    int ah, al, bh, bl;
-    fx_split(a[i], ah, al);
-    fx_split(b[i], bh, bl);
-    cross = fx_madhi(ah, bl, fx_madhi(al, bh, cross));
-    s += fx_prod(ah, bh);
-  }
-  return s + cross;
+}// the same of a >= 0 and any b, the sign apart: a stream and its reverse have
+// the same products
+FX_HD fx64 fx_smul(fx64 a, fx64 b) {
+  const fx64 s = b >> 63, t = fx_umul(a, (b ^ s) - s);
+  return (t ^ s) - s;
 }
 
 FX_HD int fx_clz64(fxu64 x) {   // x > 0
@@ -221,12 +226,29 @@ FX_HD fx64 fx_entropy(const FxConsts& C, fx64 lam, int ls) {
   return lam;
 }
 
-// Twice the Roe flux per unit area of face states L, R (rho Q64, velocity
-// Q64, p Q71) along n (Q62): mass and momentum Q65, energy Q69.  ls: the
-// face's format of the eigenvalues over c~ (Q(56 + ls), 3..6).  Returns
-// nonzero when a quantity has left its range (the flux is then not to be
-// used): |mass| < 0.166, |momentum| < 1/32, |energy| < 1/256, so that the
-// intermediate sums cannot have wrapped unnoticed.
+// What the flux is made of: density and pressure of both sides (rho Q64, p
+// Q71), |u|^2 of both and |u_R - u_L|^2 (Q64) on the face's scales; normal
+// velocities (Q(64 + kn)) and the jump of p (Q(71 + kn)) on theirs.  ls: the
+// face's format of the eigenvalues over c~ (Q(56 + ls), 3..6).
+struct FxFace {
+  fx64 rL, rR, pL, pR, qL, qR, e, VnL, VnR, dp;
+  int kn, ls;
+};
+// Twice the flux per unit area in four numbers: the mass flux M (Q(65 + kn)),
+// the factor G of u_R - u_L (Q(65 + kn)), the dissipative pressure X (Q(67 + kn)) and
+// the energy flux E (Q(69 + kn)); the momentum flux is M u_L + G (u_R - u_L) +
+// n (p_L + p_R + X).  With the entropy fix on every eigenvalue, where |lambda_2|
+// does not get small with Vn~, they are without the waves of that eigenvalue,
+// a2 = l2 dr - t2 and a3 = l2 rt, and its parts follow: l2 (Q(64 + kl)), t2 (Q(65 + kn)),
+// rt (Q64) and beta (Q62).
+struct FxFlux {
+  fx64 M, G, X, E, l2, t2, rt, beta;
+  int kl;
+};
+
+// Returns nonzero when a quantity has left its range (the flux is then not to
+// be used): |M| < 0.166, |G| < 3/16, |E| < 1/256, so that the intermediate
+// sums cannot have wrapped unnoticed.
 //
 // The same flux as roe_flux's, regrouped: with m = rho Vn of the two sides,
 // D0 = a1 + a5 + a2, beta the weight of R in the Roe averages, du = u_R - u_L,
@@ -234,24 +256,18 @@ FX_HD fx64 fx_entropy(const FxConsts& C, fx64 lam, int ls) {
 //   F_mom  = F_mass u_L + (m_R - beta D0 - a3) du + n (p_L + p_R - d51 + a3 dVn)
 //   F_en   = (F_mass + a2) h_L + (m_R - beta a15) dh - d51 Vn~ - a2 q~ - a3 (u~.du - Vn~ dVn)
 // and c~^2 = (gamma-1)(H_L + beta dH + beta (1-beta) |du|^2/2), H = c^2/(gamma-1):
-// two products per momentum component, and no cancelling h~ - |u~|^2/2.
-FX_HD unsigned fx_roe(const FxConsts& C, const fx64 L[5], const fx64 R[5], const fx64 n[3], int ls, bool fix_all,
-                      fx64 F[5]) {
-  const fx64 rL = L[0], rR = R[0], pL = L[4], pR = R[4];
-  const fx64 VnL = fx_dot3(n, L + 1) << 2, VnR = fx_dot3(n, R + 1) << 2;   // Q64
-  const fx64 mL = fx_mul(rL, VnL), mR = fx_mul(rR, VnR);                   // Q64
+// no cancelling h~ - |u~|^2/2.
+FX_HD unsigned fx_roe(const FxConsts& C, const FxFace& f, bool fix_all, FxFlux& F) {
+  const fx64 rL = f.rL, rR = f.rR, VnL = f.VnL, VnR = f.VnR, qL = f.qL, qR = f.qR, e = f.e;
+  const int kn = f.kn < 63 ? f.kn : 63, ls = f.ls;       // kn as a shift
+  const fx64 mL = fx_smul(rL, VnL), mR = fx_smul(rR, VnR);                 // Q(64 + kn)
   const fx64 dVn = VnR - VnL;
   // 1/sqrt(rho): sqrt(rho) (Q63), 1/rho (Q59)
   const fx64 yL = fx_rsqrt(rL), yR = fx_rsqrt(rR);
   const fx64 sL = fx_umul(rL, yL) << 2, sR = fx_umul(rR, yR) << 2;
   // H = gamma/(gamma-1) p/rho, Q66
-  const fx64 HL = fx_umul(fx_umul(pL, fx_umul(yL, yL) << 1) << 4, C.K);
-  const fx64 HR = fx_umul(fx_umul(pR, fx_umul(yR, yR) << 1) << 4, C.K);
-  // |u|^2, |du|^2 (Q64); their halves are Q65
-  const fx64 du[3] = {R[1] - L[1], R[2] - L[2], R[3] - L[3]};
-  const fx64 qL = fx_sqr(L[1]) + fx_sqr(L[2]) + fx_sqr(L[3]);
-  const fx64 qR = fx_sqr(R[1]) + fx_sqr(R[2]) + fx_sqr(R[3]);
-  const fx64 e = fx_sqr(du[0]) + fx_sqr(du[1]) + fx_sqr(du[2]);
+  const fx64 HL = fx_umul(fx_umul(f.pL, fx_umul(yL, yL) << 1) << 4, C.K);
+  const fx64 HR = fx_umul(fx_umul(f.pR, fx_umul(yR, yR) << 1) << 4, C.K);
   const fx64 dq = qR - qL, dH = HR - HL;
   // beta = sqrt(rho_R)/(sqrt(rho_L) + sqrt(rho_R)), Q62; rho~, Q64
   const fxu64 ss = (fxu64)sL + (fxu64)sR;                // Q63, 1/2 .. sqrt 2
@@ -271,54 +287,54 @@ FX_HD unsigned fx_roe(const FxConsts& C, const fx64 L[5], const fx64 R[5], const
   const fx64 yc = fx_rsqrt(c2 << z);
   const fx64 ic = ish >= 0 ? yc >> ish : yc << -ish;
   const fx64 c = fx_umul(c2, ic) << 4;                   // Q60 -> Q64
-  const fx64 Vnt = VnL + (fx_mul(beta << 1, dVn) << 1);
-  const fx64 t1 = Vnt - c, t5 = Vnt + c;
-  const fx64 l1 = t1 < 0 ? -t1 : t1, l5 = t5 < 0 ? -t5 : t5;
-  fx64 l2 = Vnt < 0 ? -Vnt : Vnt;
+  const fx64 Vnt = VnL + (fx_mul(beta << 1, dVn) << 1);  // Q(64 + kn)
+  const fxu64 an = fx_abs(Vnt);
+  const fx64 Vc = Vnt >> kn, ac = (fx64)(an >> kn);      // Q64
   // eigenvalues over c~, Q(56 + ls): the scales keep them below 2^(7 - ls), ls = 3..6
-  const fx64 k1 = fx_entropy(C, fx_umul(l1, ic) << ls, ls), k5 = fx_entropy(C, fx_umul(l5, ic) << ls, ls);
-  fx64 k2 = fx_umul(l2, ic) << ls;
-  if (fix_all && k2 < (C.eta >> (6 - ls))) {
-    k2 = fx_entropy(C, k2, ls);
-    l2 = fx_umul(k2, c) << (8 - ls);                      // Q(56 + ls) -> Q64
-  }
+  const fx64 k1 = fx_entropy(C, fx_umul((fx64)fx_abs(Vc - c), ic) << ls, ls);
+  const fx64 k5 = fx_entropy(C, fx_umul((fx64)fx_abs(Vc + c), ic) << ls, ls);
+  fx64 k2 = fx_umul(ac, ic) << ls;
   // wave strengths: P = dp/c~, kap = rho~ dVn
-  const fx64 dp = pR - pL, dr = rR - rL;
-  const fx64 P = fx_mul(dp, ic) << 1;                    // Q63 -> Q64
-  const fx64 kap = fx_mul(rt, dVn);                      // Q64
-  const fx64 a1 = fx_mul(k1, P - kap), a5 = fx_mul(k5, P + kap);        // x Q65 -> Q(57 + ls)
-  const fx64 t2 = fx_mul(k2, P << 2);                                   // Q(58 + ls)
-  const fx64 a3 = fx_mul(l2, rt) << 1;                                  // Q65
-  unsigned wild = (fx_mag(a1) | fx_mag(a5) | (fx_mag(t2) >> 1)) >> (19 + ls);   // each below 1/64
+  const fx64 P = fx_mul(f.dp, ic) << 1;                  // Q(63 + kn) -> Q(64 + kn)
+  const fx64 kap = fx_mul(rt, dVn);                      // Q(64 + kn)
+  const fx64 a1 = fx_smul(k1, P - kap), a5 = fx_smul(k5, P + kap);      // x Q65 -> Q(57 + ls + kn)
+  unsigned wild = (fx_mag(a1) | fx_mag(a5)) >> (20 + ls);               // each below 1/32
   wild |= fx_mag(c) >> 29;                                              // c~ below 1/8
-  const fx64 A2 = (fx_mul(l2, dr) << 1) - (t2 << (7 - ls));             // Q65 from here
-  const fx64 a15 = (a1 + a5) << (8 - ls), a51 = (a5 - a1) << (8 - ls);
-  const fx64 M1 = ((mL + mR) << 1) - a15, F0 = M1 - A2;
-  const fx64 D0 = a15 + A2;
-  const fx64 d51 = fx_mul(a51, c << 2);                                 // Q67
-  const fx64 Pi = ((pL >> 4) + (pR >> 4)) - d51 + (fx_mul(a3, dVn) << 2);   // Q67
-  const fx64 mR1 = mR << 1;
-  const fx64 G = mR1 - (fx_mul(beta << 1, D0) << 1) - a3;
-  // each product is rounded down: one unit on average, given back unless the
-  // sum is zero (a velocity that is zero everywhere stays zero)
-  F[0] = F0;
-  wild |= fx_mag(F0) > 0x54fdf3b5u || fx_mag(G) > 0x5fffffffu;
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    const fx64 w = fx_mul(F0, L[1 + i]) + fx_mul(G, du[i]) + fx_mul(n[i], Pi);
-    F[1 + i] = w ? w + 3 : 0;
-    wild |= fx_mag(F[1 + i]) >> 28;
+  const fx64 a15 = (a1 + a5) << (8 - ls), a51 = (a5 - a1) << (8 - ls);  // Q(65 + kn) from here
+  const bool fixed = fix_all && k2 < (C.eta >> (6 - ls));
+  if (fixed) k2 = fx_entropy(C, k2, ls);
+  const fx64 t2 = fx_mul(k2, P << 2);                                   // Q(58 + ls + kn)
+  wild |= (fx_mag(t2) >> 1) >> (19 + ls);                               // below 1/64
+  fx64 A2 = 0, a3 = 0;
+  if (fix_all) {
+    F.l2 = fixed ? fx_umul(k2 << (6 - ls), c) << 2 : (fx64)an;          // Q62 -> Q64
+    F.kl = fixed ? 0 : f.kn;
+    F.t2 = t2 << (7 - ls);
+    F.rt = rt;
+    F.beta = beta;
+  } else {
+    A2 = (fx_mul((fx64)an, rR - rL) << 1) - (t2 << (7 - ls));
+    a3 = fx_mul((fx64)an, rt) << 1;
   }
-  // energy, Q69
+  const fx64 M1 = ((mL + mR) << 1) - a15;
+  const fx64 D0 = a15 + A2;
+  const fx64 d51 = fx_mul(a51, c << 2);                                 // Q(67 + kn)
+  const fx64 mR1 = mR << 1;
+  F.M = M1 - A2;
+  F.X = (fx_mul(a3, dVn) << 2 >> kn) - d51;
+  F.G = mR1 - (fx_mul(beta << 1, D0) << 1) - a3;
+  wild |= fx_mag(F.M) > 0x54fdf3b5u || fx_mag(F.G) > 0x5fffffffu;
+  // energy, Q(69 + kn)
   const fx64 hL = (HL + 2 * qL) << 2, dh = (dH + 2 * dq) << 2;          // Q68
-  const fx64 qt = (qL + (fx_mul(beta << 1, dq) << 1) - b2) << 3;        // q~, Q65 -> Q68
-  const fx64 uw = (dq - e) + 2 * be;                                    // u~.du, Q65
-  const fx64 ud = (uw << 1) - (fx_mul(Vnt, dVn) << 2);                  // u~.du - Vn~ dVn, Q66
   const fx64 G4 = mR1 - (fx_mul(beta << 1, a15) << 1);
-  const fx64 w = fx_mul(M1, hL) + fx_mul(G4, dh) - fx_mul(d51 << 2, Vnt) - fx_mul(A2, qt) -
-                 (fx_mul(a3 << 1, ud) << 1);
-  F[4] = w ? w - 1 : 0;
-  return wild | (fx_mag(F[4]) >> 29);
+  F.E = fx_smul(hL, M1) + fx_mul(G4, dh) - (fx_mul(d51 << 2, Vnt) >> kn);
+  if (!fix_all) {
+    const fx64 qt = (qL + (fx_mul(beta << 1, dq) << 1) - b2) << 3;      // q~, Q65 -> Q68
+    const fx64 uw = (dq - e) + 2 * be;                                  // u~.du, Q65
+    const fx64 ud = (uw << 1) - ((fx_mul(Vnt, dVn) >> kn) >> kn << 2);  // u~.du - Vn~ dVn, Q66
+    F.E -= fx_smul(qt, A2) + (fx_smul(a3 << 1, ud) << 1);
+  }
+  return wild | (fx_mag(F.E) >> 29);
 }
 
 // ---------------------------------------------------------------------------
@@ -369,6 +385,7 @@ FX_HD float fx_approx(int h) {
 
 struct FxScale {
   int mr, mv, ls;
+  float ic;      // an upper bound of 1/c^ of both sides
 };
 // The face's scales from its two states; false when they do not fit
 FX_HD bool fx_scale(const FxConsts& C, const double VL[5], const double VR[5], FxScale& S) {
@@ -403,31 +420,42 @@ FX_HD bool fx_scale(const FxConsts& C, const double VL[5], const double VR[5], F
   S.ls = uu < 0.97f * c2 ? 6 : (uu < 8.8f * c2 ? 5 : (uu < 48.0f * c2 ? 4 : 3));
   // 1/c~ below 120 (Q56), and dp/c~ <= max p^ / min c^ < 0.12 (rho^ < 1/2)
   const float s2 = fx_asfloat((127 - 2 * S.mv) << 23), T = (tL > tR ? tL : tR) * s2;
+  S.ic = fx_rsqrtf(c2 * s2) * 1.0001f;
   return ok && uu < 220.0f * c2 && c2 * s2 > 7.0e-5f && T * T < 0.0575f * (c2 * s2);
+}
+
+// The scale of what is proportional to the normal velocities or the jumps, 2^-kn
+// of the face's: Vn^ < 2^-4-kn, rho^ |dVn^| and |dp^|/c^ < 2^-6-kn.  dn: |dVn| in
+// Q(64 + kv), at the scale 2^-kv of Vn alone; dp: |dp| in Q(71 + kp).
+FX_HD int fx_scale_n(const FxScale& S, int kv, fxu64 dn, int kp, fxu64 dp) {
+  int k = kv;
+  if (dn) {
+    const int j = kv + fx_clz64(dn) - 5;
+    k = k < j ? k : j;
+  }
+  if (dp) {
+    const int z = fx_clz64(dp);
+    const float f = fx_u2f((unsigned)((dp << z) >> 32)) * S.ic;
+    const int j = 33 + z + kp - ((fx_asint(f) >> 23) - 126);
+    k = k < j ? k : j;
+  }
+  return k < 0 ? 0 : k;
 }
 
 // binary64 value times 2^64 / 2^m (c = 1021 + m) truncated: the significand at
 // bit 62 moved right by c - E; the scales keep the shift non-negative
-FX_HD fx64 fx_convert(double x, int c) {
+FX_HD fxu64 fx_magnitude(double x, int c) {
   const int hi = fx_hi(x);
   const unsigned lo = fx_lo(x);
   const fxu64 M = ((fxu64)(((((unsigned)hi & 0xfffffu) | 0x100000u) << 10) | (lo >> 22)) << 32) | (lo << 10);
-  int r = c - ((hi >> 20) & 0x7ff);
-  r = r > 63 ? 63 : r;
-  const fx64 v = (fx64)(M >> r);
-  const fx64 sg = (fx64)(hi >> 31);
-  return (v ^ sg) - sg;
+  const unsigned r = (unsigned)(c - ((hi >> 20) & 0x7ff));
+  return M >> (r > 63u ? 63u : r);
 }
-
-// x 2^e rounded to nearest (x a fixed-point sum, the result a normal number or zero)
-FX_HD double fx_to_double(fx64 x, int e) {
-#ifdef __CUDA_ARCH__
-  const double d = __ll2double_rn(x);
-  return __hiloint2double(x ? __double2hiint(d) + (e << 20) : 0, __double2loint(d));
-#else
-  return ldexp((double)x, e);
-#endif
+FX_HD fx64 fx_sign(fxu64 v, double x) {
+  const fx64 sg = (fx64)(fx_hi(x) >> 31);
+  return ((fx64)v ^ sg) - sg;
 }
+FX_HD fx64 fx_convert(double x, int c) { return fx_sign(fx_magnitude(x, c), x); }
 
 FX_HD double fx_double(int hi, unsigned lo) {
 #ifdef __CUDA_ARCH__
@@ -438,6 +466,18 @@ FX_HD double fx_double(int hi, unsigned lo) {
   __builtin_memcpy(&d, &b, 8);
   return d;
 #endif
+}
+
+// x 2^e rounded to nearest (the result a normal number or zero).  On the
+// integer units: the conversion instruction is held by the FP64 unit (five of
+// them a face, 128^3 RK step 4.70 against 4.56 ms).
+FX_HD double fx_to_double(fx64 x, int e) {
+  const fxu64 H = fx_abs(x);
+  const int z = fx_clz64(H | 1);
+  const fxu64 N = H << z;
+  const fxu64 b = (N >> 11) + ((N >> 10) & 1) + ((fxu64)(unsigned)(e + 1085 - z) << 52);
+  const int sg = (int)(x >> 32) & (int)0x80000000;
+  return fx_double(H ? (int)(b >> 32) | sg : 0, H ? (unsigned)b : 0u);
 }
 
 // 2^30 / s' for s' = (2^32 sh + sl) / 2^64 in [1/2, 1): 32 bits (the hardware's
@@ -527,35 +567,50 @@ FX_HD double fx_vanleer_half(double a, double b) {
 }
 
 // Roe flux times the area A of the states VL, VR along the unit normal n in
-// `out`; false (out not written) when the face does not fit.  In the stage
-// kernel it took the 128^3 curvilinear block's RK step from 10.83 to 5.83 ms
-// (tile 16x8), the 64-block batch's from 79.6 to 49.2 ms; the binary64
-// pipe, which it leaves to the slopes, the sums and the update, was the
-// bound before.
+// `out`; false (out not written) when the face does not fit.
 FX_HD bool fx_roe_flux(const FxConsts& C, const double VL[5], const double VR[5], double nx, double ny, double nz,
                        double A, bool fix_all, double out[5]) {
-  FxScale S;
-  if (!fx_scale(C, VL, VR, S)) return false;
-  const int ah = fx_hi(A);
-  if (!((unsigned)ah - (823u << 20) < (400u << 20))) return false;   // 2^-200 .. 2^200
-  fx64 L[5], R[5], n[3], F[5];
-  const int cr = 1021 + S.mr, cv = 1021 + S.mv, cp = 1014 + S.mr + 2 * S.mv;
-  L[0] = fx_convert(VL[0], cr);
-  R[0] = fx_convert(VR[0], cr);
-#pragma unroll
-  for (int i = 1; i < 4; ++i) {
-    L[i] = fx_convert(VL[i], cv);
-    R[i] = fx_convert(VR[i], cv);
-  }
-  L[4] = fx_convert(VL[4], cp);
-  R[4] = fx_convert(VR[4], cp);
   // |n_i| <= 1 up to rounding: a NaN or a larger value does not fit
   const int nm = (fx_hi(nx) & 0x7fffffff) > (fx_hi(ny) & 0x7fffffff) ? fx_hi(nx) & 0x7fffffff : fx_hi(ny) & 0x7fffffff;
   if ((nm > (fx_hi(nz) & 0x7fffffff) ? nm : fx_hi(nz) & 0x7fffffff) >= (1024 << 20)) return false;
-  n[0] = fx_convert(nx, 1023);
-  n[1] = fx_convert(ny, 1023);
-  n[2] = fx_convert(nz, 1023);
-  if (fx_roe(C, L, R, n, S.ls, fix_all, F)) return false;
+  const int ah = fx_hi(A);
+  if (!((unsigned)ah - (823u << 20) < (400u << 20))) return false;   // 2^-200 .. 2^200
+  FxScale S;
+  if (!fx_scale(C, VL, VR, S)) return false;
+  const double VnL = fma(nx, VL[1], fma(ny, VL[2], nz * VL[3])), VnR = fma(nx, VR[1], fma(ny, VR[2], nz * VR[3]));
+  FxFace f;
+  const int cr = 1021 + S.mr, cv = 1021 + S.mv, cp = 1014 + S.mr + 2 * S.mv;
+  // (2^-400 of the face's scale is zero)
+  const int hn = (fx_hi(VnL) & 0x7fffffff) > (fx_hi(VnR) & 0x7fffffff) ? fx_hi(VnL) & 0x7fffffff : fx_hi(VnR) & 0x7fffffff;
+  int kv = S.mv - 4 - ((hn >> 20) - 1022);
+  if (kv < -2) return false;   // |Vn^| above 1/4: no unit normal
+  kv = kv < 0 ? 0 : (kv < 400 ? kv : 400);
+  f.VnL = fx_convert(VnL, cv - kv);
+  f.VnR = fx_convert(VnR, cv - kv);
+  const int em = (fx_hi(VL[4]) > fx_hi(VR[4]) ? fx_hi(VL[4]) : fx_hi(VR[4])) >> 20, kp = cp - em;
+  f.pL = (fx64)fx_magnitude(VL[4], em);
+  f.pR = (fx64)fx_magnitude(VR[4], em);
+  f.dp = f.pR - f.pL;
+  f.kn = fx_scale_n(S, kv, fx_abs(f.VnR - f.VnL), kp, fx_abs(f.dp));
+  f.VnL >>= kv - f.kn < 63 ? kv - f.kn : 63;
+  f.VnR >>= kv - f.kn < 63 ? kv - f.kn : 63;
+  f.pL >>= kp;
+  f.pR >>= kp;
+  f.dp = f.kn > kp ? f.dp << (f.kn - kp < 63 ? f.kn - kp : 63) : f.dp >> (kp - f.kn);
+  f.ls = S.ls;
+  f.rL = (fx64)fx_magnitude(VL[0], cr);
+  f.rR = (fx64)fx_magnitude(VR[0], cr);
+  f.qL = f.qR = f.e = 0;
+#pragma unroll
+  for (int i = 1; i < 4; ++i) {
+    const fxu64 a = fx_magnitude(VL[i], cv), b = fx_magnitude(VR[i], cv);
+    f.qL += fx_usqr(a);
+    f.qR += fx_usqr(b);
+    f.e += fx_usqr(fx_abs(fx_sign(b, VR[i]) - fx_sign(a, VL[i])));
+  }
+  fix_all = fix_all && C.eta > 0;
+  FxFlux F;
+  if (fx_roe(C, f, fix_all, F)) return false;
   // the area's significand, Q63 in [1/2, 1) with its top kept from rounding
   // up to 1 (fx_split), and exponent; F is twice the flux
   const unsigned al = fx_lo(A);
@@ -563,10 +618,32 @@ FX_HD bool fx_roe_flux(const FxConsts& C, const double VL[5], const double VR[5]
   const fx64 am = (fx64)((((fxu64)(((((unsigned)ah & 0xfffffu) | 0x100000u) << 10) | (al >> 22)) << 32) | (al << 10)) >>
                          (ea - (ah >> 20)));
   const int e = ea - 1022 - 65 + S.mr + S.mv;
-  out[0] = fx_to_double(fx_mul(F[0], am), e);
-  out[1] = fx_to_double(fx_mul(F[1], am), e + S.mv);
-  out[2] = fx_to_double(fx_mul(F[2], am), e + S.mv);
-  out[3] = fx_to_double(fx_mul(F[3], am), e + S.mv);
-  out[4] = fx_to_double(fx_mul(F[4], am), e - 4 + 2 * S.mv);
+  double M = fx_to_double(fx_smul(am, F.M), e - f.kn), G = fx_to_double(fx_mul(F.G, am), e - f.kn);
+  double X = fx_to_double(fx_mul(F.X, am), e - 2 + S.mv - f.kn);
+  double E = fx_to_double(fx_smul(am, F.E), e - 4 + 2 * S.mv - f.kn);
+  const double hA = fx_double(ah - (1 << 20), al);
+  if (fix_all) {
+    const double b = fx_to_double(F.beta, -62), dVn = VnR - VnL;
+    const double l2A = fx_to_double(F.l2, S.mv - 64 - F.kl) * hA;
+    const double a2 = fma(l2A, VR[0] - VL[0], -fx_to_double(fx_mul(F.t2, am), e - f.kn));
+    const double a3 = l2A * fx_to_double(F.rt, S.mr - 64);
+    double ud = -fma(b, dVn, VnL) * dVn, q = 0.0;
+#pragma unroll
+    for (int i = 1; i < 4; ++i) {
+      const double du = VR[i] - VL[i], ut = fma(b, du, VL[i]);
+      ud = fma(ut, du, ud);
+      q = fma(ut, ut, q);
+    }
+    M -= a2;
+    G = fma(-b, a2, G) - a3;
+    X = fma(a3, dVn, X);
+    E = fma(-0.5 * a2, q, fma(-a3, ud, E));
+  }
+  const double P = fma(VL[4] + VR[4], hA, X);
+  out[0] = M;
+  out[1] = fma(nx, P, fma(M, VL[1], G * (VR[1] - VL[1])));
+  out[2] = fma(ny, P, fma(M, VL[2], G * (VR[2] - VL[2])));
+  out[3] = fma(nz, P, fma(M, VL[3], G * (VR[3] - VL[3])));
+  out[4] = E;
   return true;
 }
