@@ -514,7 +514,8 @@ FX_HD fxu64 fx_round(fxu64 H, int e) {
 }
 
 // n / d for a finite d > 0, within 0.65 units in the last place; a quotient
-// below the normal range is 0, above it infinite, of a non-finite n NaN
+// below the normal range is 0, above it infinite, of a non-finite n or a
+// subnormal d NaN
 FX_HD double fx_div(double n, double d) {
   const int hn = fx_hi(n), hd = fx_hi(d);
   const unsigned ln = fx_lo(n), ld = fx_lo(d);
@@ -528,7 +529,7 @@ FX_HD double fx_div(double n, double d) {
   const int e = en - ed + 1024;
   const fxu64 b = fx_round(H, e);
   const int sg = hn & (int)0x80000000;
-  const bool nan = en == 2047 || ed == 2047 || hd <= 0;
+  const bool nan = en == 2047 || ed == 2047 || hd < (1 << 20);
   const bool zero = en == 0 || e < 4;
   const bool inf = (unsigned)(b >> 52) >= 2047u;
   const int hi = nan ? 0x7ff80000 : (zero ? sg : (inf ? sg | 0x7ff00000 : sg | (int)(b >> 32)));
@@ -561,7 +562,10 @@ FX_HD double fx_vanleer_half(double a, double b) {
   const fxu64 H = fx_quot((fxu64)fx_umul((fx64)A, (fx64)B), r, e2);     // product in [2^60, 2^62)
   // h = H 2^(n + ea + eb - em - 1085)
   const fxu64 bits = fx_round(H, en + 1 + n);
-  const bool zero = (ha ^ hb) < 0 || em < 923 || en < 64;
+  // a NaN comes through whatever the signs, an infinity with a number of its sign gives one
+  const int ma = ha & 0x7fffffff, mb = hb & 0x7fffffff;
+  const bool nan = (ma > mb ? ma : mb) > 0x7ff00000;
+  const bool zero = !nan && ((ha ^ hb) < 0 || em < 923 || en < 64);
   const int hh = (int)(bits >> 32) | (ha & (int)0x80000000);
   return fx_double(zero ? 0 : (em == 2047 ? 0x7ff80000 : hh), zero ? 0u : (unsigned)bits);
 }
