@@ -466,6 +466,21 @@ int fv_check_rcp64(const double* x_dev, int64_t n, double* out_dev, void* stream
  * IEEE sqrt(x[i]).  Arguments, stream and errors as fv_check_rcp64. */
 int fv_check_sqrt64(const double* x_dev, int64_t n, double* out_dev, void* stream);
 
+/* Test support for the face code's other operations on the device: op 0 the
+ * integer quotient a / b, 1 the integer half-slope a b / (a + b), and of a and
+ * b split into double-float pairs 2 the quotient, 3 the square root of a, 4 the
+ * half-slope, 5 the reciprocal of a.  out_dev[2i], out_dev[2i+1]: the result's
+ * two parts (binary64 results: the second is zero).  Asynchronous on `stream`;
+ * FV_ERR_INVALID_ARG for NULL pointers, n <= 0 or another op. */
+int fv_check_face_op(int op, const double* a_dev, const double* b_dev, int64_t n, double* out_dev, void* stream);
+
+/* Test support for the binary64 form's fixed-point Roe flux on the device: n
+ * faces of 14 doubles (left and right (rho, u, v, w, p), unit normal, area) in,
+ * 6 out (1 if the face fits the fixed point, else 0; the five fluxes).
+ * Asynchronous on `stream`; errors as fv_check_face_op. */
+int fv_check_roe64(const double* faces_dev, int64_t n, double gamma, double harten, int fix_all, double* out_dev,
+                   void* stream);
+
 /* ---------------------------------------------------------------------------
  * Allocation-free residual norms.  The paper has no counterpart: this entry
  * point exists for callers that must not allocate device memory while they

@@ -25,7 +25,7 @@ EXPORTS = ("fv_config_default", "fv_create_blocks", "fv_destroy", "fv_last_error
            "fv_adjoint_vjp", "fv_autotune", "fv_get_launch", "fv_set_boundaries", "fv_set_monitor",
            "fv_monitor_norms", "fv_stage_state", "fv_set_state_staged", "fv_graph_count",
            "fv_probe_alu_rates", "fv_set_halo", "fv_halo_size", "fv_halo_pack", "fv_halo_unpack",
-           "fv_check_rcp64", "fv_check_sqrt64", "fv_set_adjoint_arith")
+           "fv_check_rcp64", "fv_check_sqrt64", "fv_check_face_op", "fv_check_roe64", "fv_set_adjoint_arith")
 
 
 class FvError(RuntimeError):
@@ -115,6 +115,10 @@ def load_library(path: Optional[str] = None):
     L.fv_check_rcp64.restype = i32
     L.fv_check_sqrt64.argtypes = [vp, i64, vp, vp]
     L.fv_check_sqrt64.restype = i32
+    L.fv_check_face_op.argtypes = [i32, vp, vp, i64, vp, vp]
+    L.fv_check_face_op.restype = i32
+    L.fv_check_roe64.argtypes = [vp, i64, ctypes.c_double, ctypes.c_double, i32, vp, vp]
+    L.fv_check_roe64.restype = i32
     L.fv_set_halo.argtypes = [vp, ctypes.POINTER(fv_connection), i32, ctypes.POINTER(fv_connection), i32]
     L.fv_set_halo.restype = i32
     L.fv_halo_size.argtypes = [vp, i32]
@@ -203,6 +207,33 @@ def check_sqrt64(x):
     """(face-code square root, IEEE sqrt(x)) of a float64 CUDA tensor x, as a
     (n, 2) tensor (fv_check_sqrt64)."""
     return _check_arith("fv_check_sqrt64", x)
+
+
+FACE_OPS = {"quotient": 0, "half_slope": 1, "df64_quotient": 2, "df64_sqrt": 3, "df64_half_slope": 4, "df64_rcp": 5}
+
+
+def check_face_op(op, a, b):
+    """One of FACE_OPS on float64 CUDA tensors: the results' two parts, as a
+    (n, 2) tensor (fv_check_face_op)."""
+    import torch
+    L = load_library()
+    out = torch.empty((a.numel(), 2), dtype=torch.float64, device=a.device)
+    rc = L.fv_check_face_op(FACE_OPS[op], _ptr(a), _ptr(b), min(a.numel(), b.numel()), out.data_ptr(), _stream(None))
+    if rc != FV_OK:
+        raise FvError(rc, "fv_check_face_op failed")
+    return out
+
+
+def check_roe64(faces, gamma=1.4, harten=0.1, fix_all=0):
+    """The fixed-point Roe flux of (n, 14) faces on the device: (n, 6), the
+    first column 1 where the face fits (fv_check_roe64)."""
+    import torch
+    L = load_library()
+    out = torch.empty((faces.numel() // 14, 6), dtype=torch.float64, device=faces.device)
+    rc = L.fv_check_roe64(_ptr(faces), faces.numel() // 14, gamma, harten, int(fix_all), out.data_ptr(), _stream(None))
+    if rc != FV_OK:
+        raise FvError(rc, "fv_check_roe64 failed")
+    return out
 
 
 class Solver:

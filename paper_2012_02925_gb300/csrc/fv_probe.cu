@@ -13,7 +13,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/fvgb.h"
-#include "fv_arith.cuh"
+#include "fv_face.cuh"
 
 namespace {
 
@@ -182,4 +182,58 @@ extern "C" int fv_check_rcp64(const double* x_dev, int64_t n, double* out_dev, v
 
 extern "C" int fv_check_sqrt64(const double* x_dev, int64_t n, double* out_dev, void* stream) {
   return arith_check((const void*)arith_check_kernel<true>, x_dev, n, out_dev, stream);
+}
+
+// ---------------------------------------------------------------------------
+// the fixed-point and double-float face operations on the device, for tests
+// ---------------------------------------------------------------------------
+namespace {
+__device__ df64 probe_pair(double x) { return fv_d2df(x); }
+
+__global__ void face_op_kernel(int op, const double* __restrict__ a, const double* __restrict__ b, long long n,
+                               double* __restrict__ out) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double x = a[i], y = b[i];
+    double hi = 0.0, lo = 0.0;
+    if (op == 0) hi = fx_div(x, y);
+    else if (op == 1) hi = fx_vanleer_half(x, y);
+    else {
+      const df64 u = probe_pair(x), v = probe_pair(y);
+      const df64 r = op == 2 ? u / v : (op == 3 ? df_sqrt(u) : (op == 4 ? vanleer_half<df64>(u, v) : df_rcp(u)));
+      hi = (double)r.hi;
+      lo = (double)r.lo;
+    }
+    out[2 * i] = hi;
+    out[2 * i + 1] = lo;
+  }
+}
+
+__global__ void face_roe_kernel(const FxConsts C, int fix_all, const double* __restrict__ x, long long n,
+                                double* __restrict__ out) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    double L[5], R[5], F[5] = {0, 0, 0, 0, 0};
+    const double* f = x + 14 * i;
+    for (int m = 0; m < 5; ++m) {
+      L[m] = f[m];
+      R[m] = f[5 + m];
+    }
+    out[6 * i] = C.on && fx_roe_flux(C, L, R, f[10], f[11], f[12], f[13], fix_all != 0, F) ? 1.0 : 0.0;
+    for (int m = 0; m < 5; ++m) out[6 * i + 1 + m] = F[m];
+  }
+}
+
+unsigned check_grid(long long n) { return (unsigned)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096); }
+}  // namespace
+
+extern "C" int fv_check_face_op(int op, const double* a_dev, const double* b_dev, int64_t n, double* out_dev, void* stream) {
+  if (!a_dev || !b_dev || !out_dev || n <= 0 || op < 0 || op > 5) return FV_ERR_INVALID_ARG;
+  face_op_kernel<<<check_grid(n), 256, 0, (cudaStream_t)stream>>>(op, a_dev, b_dev, n, out_dev);
+  return cudaGetLastError() == cudaSuccess ? FV_OK : FV_ERR_CUDA;
+}
+
+extern "C" int fv_check_roe64(const double* faces_dev, int64_t n, double gamma, double harten, int fix_all, double* out_dev,
+                              void* stream) {
+  if (!faces_dev || !out_dev || n <= 0) return FV_ERR_INVALID_ARG;
+  face_roe_kernel<<<check_grid(n), 256, 0, (cudaStream_t)stream>>>(fx_consts(gamma, harten), fix_all, faces_dev, n, out_dev);
+  return cudaGetLastError() == cudaSuccess ? FV_OK : FV_ERR_CUDA;
 }
