@@ -163,17 +163,18 @@ __device__ __forceinline__ float fv_rcp(float x) {
 }
 
 // a / b: quotient estimate q1 of the high parts, its remainder a - b q1 by
-// fused multiply-adds (the high parts' is exact up to its last bit), and the
-// correction q2.  Error as the IEEE reciprocal with a double-float remainder
-// gives (rms 3.2e-15, at most 3.2e-14 of the quotient), at 11 instructions
-// instead of 37: 128^3 double-float RK step 3.00 -> 2.73 ms, the 151x49x27
-// O-grid's 0.635 -> 0.536 ms
+// fused multiply-adds (the high parts' is exact up to its last bit), the
+// correction q2 and the correction's own remainder.  Error rms 2.6e-15, at most
+// 2.8e-14 of the quotient (an IEEE reciprocal with a double-float remainder gives
+// 3.2e-15 and 3.2e-14; without the last two operations here 3.2e-15 and 3.4e-14),
+// at 13 instructions instead of 37
 FV_HD df64 operator/(df64 a, df64 b) {
   const float r = fv_rcp(b.hi);
   const float q1 = FMUL(a.hi, r);
   const float e = FFMA(-q1, b.hi, a.hi);
-  const float q2 = FMUL(FFMA(-q1, b.lo, FADD(e, a.lo)), r);
-  return quick_two_sum(q1, q2);
+  const float rem = FFMA(-q1, b.lo, FADD(e, a.lo));
+  const float q2 = FMUL(rem, r);
+  return quick_two_sum(q1, FFMA(FFMA(-q2, b.hi, rem), r, q2));
 }
 FV_HD df64 df_rcp(df64 b) {
   const float r = fv_rcp(b.hi);
@@ -181,8 +182,9 @@ FV_HD df64 df_rcp(df64 b) {
 }
 
 // square root: the hardware's approximate reciprocal square root, one coupled
-// Newton step for s ~ sqrt(a.hi) and h ~ 1/(2 s), then the remainder a - s^2
-// (error as from the IEEE binary32 root: rms 1.4e-15, at most 1.4e-14)
+// Newton step for s ~ sqrt(a.hi) and h ~ 1/(2 s), then the remainder a - s^2 with
+// the rounding of its sum (error rms 1.2e-15, at most 1.2e-14; from an IEEE binary32
+// root and reciprocal 1.5e-15 and 1.3e-14, without the sum's rounding 1.5e-15 and 1.5e-14)
 FV_HD df64 df_sqrt(df64 a) {
   if (!(a.hi > 0.0f)) return mk(a.hi == 0.0f ? 0.0f : __int_as_float(0x7fc00000), 0.0f);
   float y;
@@ -190,8 +192,8 @@ FV_HD df64 df_sqrt(df64 a) {
   const float s0 = FMUL(a.hi, y), h0 = FMUL(0.5f, y);
   const float d = FFMA(-s0, h0, 0.5f);
   const float s = FFMA(s0, d, s0), h = FFMA(h0, d, h0);
-  const float e = FADD(FFMA(-s, s, a.hi), a.lo);
-  return quick_two_sum(s, FMUL(e, h));
+  const df64 e = two_sum(FFMA(-s, s, a.hi), a.lo);
+  return quick_two_sum(s, FFMA(e.hi, h, FMUL(e.lo, h)));
 }
 FV_HD df64 df_abs(df64 a) { return a.hi < 0.0f ? -a : a; }
 FV_HD bool operator<(df64 a, df64 b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }

@@ -111,24 +111,15 @@ __device__ __forceinline__ void prim_from_cons(const CC& C, const T q[5], T V[5]
 // (rounding noise of a quantity that is zero, e.g. a transverse velocity):
 // zero slope, as the oracle's guarded ratio gives to within 2e-30; it also
 // keeps the binary32 reciprocal of a subnormal sum from overflowing.
+// (Double-float: with product and sum left unnormalised before the quotient the
+// slope's error is a tenth to a third larger, 3.5e-15 rms and 4.0e-14 at most instead
+// of 3.1e-15 and 3.0e-14; 128^3 RK step with that and without the quotient's and the
+// root's last corrections 2.50 instead of 2.61 ms.)
 template <class T>
 __device__ __forceinline__ T vanleer_half(T a, T b) {
   using S = Sc<T>;
   // binary64: on the integer units
   if constexpr (std::is_same<T, double>::value) return fx_vanleer_half(a, b);
-  // double-float: product and sum of the same sign feed the quotient only, so
-  // neither is renormalised
-  if constexpr (std::is_same<T, df64>::value) {
-    const float p = FMUL(a.hi, b.hi);
-    float pe = FFMA(a.hi, b.hi, -p);
-    pe = FFMA(a.hi, b.lo, pe);
-    pe = FFMA(a.lo, b.hi, pe);
-    df64 s = two_sum(a.hi, b.hi);
-    s.lo = FADD(s.lo, FADD(a.lo, b.lo));
-    const df64 h = mk(p, pe) / s;
-    const bool on = p > 0.0f && fabsf(s.hi) > 1e-30f;
-    return mk(on ? h.hi : 0.0f, on ? h.lo : 0.0f);
-  }
   const T p = a * b, s = a + b;
   const T h = S::div(p, s);
   return S::sel(S::pos(p) && S::above(S::abs(s), 1e-30f), h, S::c(0.0));
