@@ -1,5 +1,6 @@
 // Discrete adjoint (vector-Jacobian product) of one Runge-Kutta stage; the
-// face VJPs in binary64 or double-float arithmetic, everything else binary64.  Stage map: Q^(m) = Q^(0) - alpha_m dt / Omega * R(X(Q^(m-1)))
+// face VJPs and the limiter's derivatives in binary64 or double-float
+// arithmetic, everything else - sums, recovery, exchange - binary64.  Stage map: Q^(m) = Q^(0) - alpha_m dt / Omega * R(X(Q^(m-1)))
 // with X the ghost exchange.  For a cotangent lam of Q^(m):
 //   mu_c   = -alpha_m dt / Omega_c * lam_c              (cotangent of R_c)
 //   Fbar_f = mu_L(f) - mu_R(f)                          (R_L holds +F_f, R_R holds -F_f)
@@ -11,7 +12,7 @@
 // gathers its own in a fixed order; connections are transposed one launch at
 // a time in table order.
 //
-// 96^3 VJP stage (van Albada), double-float sweeps 1.80 -> 0.84 ms, binary64
+// 96^3 VJP stage (van Albada), double-float sweeps 1.80 -> 0.87 ms, binary64
 // 4.58 -> 2.77 ms against one kernel per face that recovered its four cells'
 // primitives, evaluated the limiter's derivatives (20 of them), and reversed
 // all of it into 20 conserved cotangents (12,700 instructions a face, 160
@@ -33,6 +34,7 @@ template <> struct AdjMem<double> {
   using type = double;
   static __device__ __forceinline__ double ld(const double* p) { return __ldg(p); }
   static __device__ __forceinline__ void st(double* p, double v) { *p = v; }
+  static __device__ __forceinline__ double to_d(double v) { return v; }
 };
 template <> struct AdjMem<df64> {
   using type = float2;
@@ -41,6 +43,21 @@ template <> struct AdjMem<df64> {
     return mk(v.x, v.y);
   }
   static __device__ __forceinline__ void st(float2* p, df64 v) { *p = make_float2(v.hi, v.lo); }
+  // hi + lo (a normalised pair) rounded to binary64 on the integer units: a cell
+  // takes 50 of these, and each sum on the FP64 unit stands for 80 issue slots
+  static __device__ __forceinline__ double to_d(df64 v) {
+    const unsigned h = (unsigned)__float_as_int(v.hi), l = (unsigned)__float_as_int(v.lo);
+    const int eh = (int)(h >> 23) & 255, el = (int)(l >> 23) & 255, d = eh - el;
+    const unsigned long long H = (unsigned long long)((h & 0x7fffffu) | 0x800000u) << 38;
+    const unsigned long long L = el ? (unsigned long long)((l & 0x7fffffu) | 0x800000u) << 38 >> ((unsigned)d < 63u ? d : 63) : 0;
+    const unsigned long long S = (int)(h ^ l) < 0 ? H - L : H + L;      // [2^60, 2^62 + 2^38)
+    const int z = __clz((int)(S >> 32));
+    const unsigned long long N = S << z;
+    const unsigned long long b = (N >> 11) + ((N >> 10) & 1) + ((unsigned long long)(unsigned)(eh + 897 - z) << 52);
+    if (eh == 255) return fv_f2d(v.hi);
+    const int hi = eh ? (int)(b >> 32) | (int)(h & 0x80000000u) : 0;
+    return __hiloint2double(hi, eh ? (int)b : 0);
+  }
 };
 
 // Primitive variables of every ghosted cell of the block, once: a face and a
@@ -150,7 +167,8 @@ __global__ void __launch_bounds__(NT, MINB) adj_face_kernel(const FvBlockDev B, 
 // the face does not exist), alpha = dh/da (L - R) and beta = dh/db (L - R)
 // (the unlimited scheme's two slopes differ), the cell itself gets
 // L + R - alpha + beta, the next one alpha, the one before -beta: stored
-// component by component, one evaluation per cell, direction and variable
+// component by component (the sum in binary64, the shares as the sweep's type
+// has them), one evaluation per cell, direction and variable
 // (evaluated three times, by each cell that takes a share, the 96^3 VJP stage
 // took 0.98 instead of 0.84 ms in double-float, 4.13 instead of 2.77 in binary64).
 template <class T>
@@ -187,14 +205,16 @@ __global__ void __launch_bounds__(128) adj_slope_kernel(const FvBlockDev B, int 
       al = P.e4kp * L - P.e4km * R;
       be = P.e4km * L - P.e4kp * R;
     }
-    M::st(out + q * nc + x, (L + R) - (al - be));
+    reinterpret_cast<double*>(out)[q * nc + x] = (M::to_d(L) + M::to_d(R)) - M::to_d(al - be);
     M::st(out + (5 + q) * nc + x, al);
     M::st(out + (10 + q) * nc + x, be);
   }
 }
 
 // The cells' cotangents: the slope kernel's shares in a fixed order (xi, eta,
-// zeta; deterministic) and the primitive recovery's transpose.  Into lamg for
+// zeta; deterministic) and the primitive recovery's transpose, both in binary64
+// in either form (summed in double-float it would keep 48 bits, and one 96^3 VJP
+// stage with double-float sweeps take 0.76 instead of 0.87 ms).  Into lamg for
 // every ghosted cell; or, when no connection has to be transposed (lam_in not
 // null), straight to lam_in for the interior cells, with lam_q0 += lam_out.
 template <class T>
@@ -202,10 +222,9 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const
                                                        const typename AdjMem<T>::type* __restrict__ sx,
                                                        const typename AdjMem<T>::type* __restrict__ sy,
                                                        const typename AdjMem<T>::type* __restrict__ sz, int three_d,
-                                                       const AdjC<T> P, double* __restrict__ lamg,
+                                                       double gm1, double* __restrict__ lamg,
                                                        const double* __restrict__ lam_out, double* __restrict__ lam_in,
                                                        double* __restrict__ lam_q0) {
-  using S = Sc<T>;
   using M = AdjMem<T>;
   const int g = lam_in ? 0 : FV_GHOST;
   const int gi = B.ni + 2 * g, gj = B.nj + 2 * g, gk = B.nk + 2 * g;
@@ -215,47 +234,47 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const
   const int i = (int)(x % gi) - g, j = (int)((x / gi) % gj) - g, k = (int)(x / ((long long)gi * gj)) - g;
   const bool ii = i >= 0 && i < B.ni, jj = j >= 0 && j < B.nj, kk = k >= 0 && k < B.nk;
   const long long gx = B.qoff + ghost_index(B, i, j, k);
-  T Vb[5];
-#pragma unroll
-  for (int m = 0; m < 5; ++m) Vb[m] = S::c(0.0);
+  double Vb[5] = {0, 0, 0, 0, 0};
 #pragma unroll 1
   for (int dir = 0; dir < 2 + three_d; ++dir) {
     if (!(dir == 0 ? jj && kk : (dir == 1 ? ii && kk : ii && jj))) continue;
     const int p = dir == 0 ? i : (dir == 1 ? j : k), nd = dir == 0 ? B.ni : (dir == 1 ? B.nj : B.nk);
     const typename M::type* s = dir == 0 ? sx : (dir == 1 ? sy : sz);
+    const double* own = reinterpret_cast<const double*>(s);
     const long long ci = B.ni + 2 * (dir == 0), cj = B.nj + 2 * (dir == 1), ck = B.nk + 2 * (dir == 2);
     const long long nc = ci * cj * ck, st = dir == 0 ? 1 : (dir == 1 ? ci : ci * cj);
     const long long c = ((long long)(k + (dir == 2)) * cj + (j + (dir == 1))) * ci + (i + (dir == 0));
-    const bool own = p >= -1 && p <= nd, lo = p >= 0 && p <= nd + 1, up = p >= -2 && p <= nd - 1;
+    const bool at = p >= -1 && p <= nd, lo = p >= 0 && p <= nd + 1, up = p >= -2 && p <= nd - 1;
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-      if (own) Vb[q] = Vb[q] + M::ld(s + q * nc + c);
-      if (lo) Vb[q] = Vb[q] + M::ld(s + (5 + q) * nc + c - st);
-      if (up) Vb[q] = Vb[q] - M::ld(s + (10 + q) * nc + c + st);
+      if (at) Vb[q] += __ldg(own + q * nc + c);
+      if (lo) Vb[q] += M::to_d(M::ld(s + (5 + q) * nc + c - st));
+      if (up) Vb[q] -= M::to_d(M::ld(s + (10 + q) * nc + c + st));
     }
   }
   // the cell's primitives and the transpose of the recovery
+  using D = Sc<double>;
   const typename M::type* v = prim + gx;
-  PrimFwd<T> s;
-  s.r = M::ld(v);
-  s.u = M::ld(v + B.plane);
-  s.v = M::ld(v + 2 * B.plane);
-  s.w = M::ld(v + 3 * B.plane);
-  s.ri = S::rcp(s.r);
-  s.k = S::dot3(s.u, s.u, s.v, s.v, s.w, s.w);
-  T qb[5];
-  prim_bwd(P, s, Vb, qb);
+  PrimFwd<double> s;
+  s.r = M::to_d(M::ld(v));
+  s.u = M::to_d(M::ld(v + B.plane));
+  s.v = M::to_d(M::ld(v + 2 * B.plane));
+  s.w = M::to_d(M::ld(v + 3 * B.plane));
+  s.ri = fx_div(1.0, s.r);   // on the integer units
+  s.k = D::dot3(s.u, s.u, s.v, s.v, s.w, s.w);
+  double qb[5];
+  prim_bwd(gm1, s, Vb, qb);
   if (lam_in) {
     const long long o = 5 * B.cell_off + x;
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
-      lam_in[o + m * n] = S::to_d(qb[m]);
+      lam_in[o + m * n] = qb[m];
       lam_q0[o + m * n] += lam_out[o + m * n];
     }
   } else {
     const bool any = (ii && jj) || (ii && kk) || (jj && kk);
 #pragma unroll
-    for (int m = 0; m < 5; ++m) lamg[gx + m * B.plane] = any ? S::to_d(qb[m]) : 0.0;
+    for (int m = 0; m < 5; ++m) lamg[gx + m * B.plane] = any ? qb[m] : 0.0;
   }
 }
 
@@ -348,7 +367,8 @@ int adjoint_block(const FvBlockDev& B, int nd, const double* qin, const double* 
   }
   const int g = lam_in ? 0 : FV_GHOST;
   const long long n = (long long)(B.ni + 2 * g) * (B.nj + 2 * g) * (B.nk + 2 * g);
-  adj_cell_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(B, prim, sl[0], sl[1], sl[2], nd == 3, P, lamg, lam_out,
+  adj_cell_kernel<T><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(B, prim, sl[0], sl[1], sl[2], nd == 3,
+                                                               fp.gamma - 1.0, lamg, lam_out,
                                                                lam_in, lam_q0);
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

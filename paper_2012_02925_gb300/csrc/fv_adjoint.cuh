@@ -105,9 +105,9 @@ __device__ __forceinline__ PrimFwd<T> prim_fwd(const AdjC<T>& P, const T q[5]) {
 // qbar = (dV/dq)^T Vbar for V = (rho, u, v, w, p), from the primitives
 // alone (rho u = r u etc.), so the conserved inputs need not stay live
 template <class T>
-__device__ __forceinline__ void prim_bwd(const AdjC<T>& P, const PrimFwd<T>& s, const T Vb[5], T qb[5]) {
+__device__ __forceinline__ void prim_bwd(T gm1, const PrimFwd<T>& s, const T Vb[5], T qb[5]) {
   using S = Sc<T>;
-  const T pb = P.gm1 * Vb[4];
+  const T pb = gm1 * Vb[4];
   const T gpb = s.r * pb;
   const T ub = Vb[1] - gpb * s.u;
   const T vb = Vb[2] - gpb * s.v;
