@@ -23,6 +23,7 @@ import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -232,17 +233,30 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(self.rows)}
 
 
+def kernel_sources():
+    """Files the fused stage kernel is compiled from: the translation units that
+    instantiate it and every header of the package they include, directly or not."""
+    d = os.path.join(ROOT, "paper_2012_02925_gb300", "csrc")
+    todo = [f for f in os.listdir(d) if f.startswith("fv_stage_") and f.endswith(".cu")]
+    seen = set()
+    while todo:
+        f = todo.pop()
+        if f in seen:
+            continue
+        seen.add(f)
+        with open(os.path.join(d, f)) as src:
+            names = re.findall(r'^\s*#\s*include\s+"([^"]+)"', src.read(), flags=re.M)
+        todo += [n for n in names if os.path.exists(os.path.join(d, n)) and os.path.dirname(n) == ""]
+    return sorted(seen)
+
+
 def kernel_hash() -> str:
-    """Hash of the sources the fused stage kernel is compiled from (its
-    template, face code, arithmetic, shared structures and the translation
-    units instantiating it): the traffic measured for it is valid while this
-    is unchanged."""
+    """Hash of kernel_sources(): the traffic measured for the stage kernel is
+    valid while this is unchanged."""
     h = hashlib.sha256()
     d = os.path.join(ROOT, "paper_2012_02925_gb300", "csrc")
-    for f in sorted(os.listdir(d)):
-        if f in ("fv_stage.cuh", "fv_face.cuh", "fv_arith.cuh", "fv_viscface.cuh", "fv_internal.h") or \
-                (f.startswith("fv_stage_") and f.endswith(".cu")):
-            h.update(open(os.path.join(d, f), "rb").read())
+    for f in kernel_sources():
+        h.update(open(os.path.join(d, f), "rb").read())
     return h.hexdigest()[:16]
 
 
