@@ -120,8 +120,6 @@ template <class T>
 __host__ __device__ constexpr bool stage_share() {
   return std::is_same<T, double>::value;
 }
-// planes in the 3-D ring: with shared slopes a pass reads planes k .. k+2
-// only, unless a slip-wall zeta face on a block's upper side reads k - 1
 // Two barriers a plane instead of three (DEEP): the plane after next is staged
 // beside the faces, and the next plane's slopes are taken beside the update,
 // which costs one more ring plane.  For the 64-cell tile, whose four resident
@@ -131,11 +129,13 @@ template <class T, int TX, int TY>
 __host__ __device__ constexpr bool stage_deep() {
   return stage_share<T>() && TX * TY <= 64;
 }
+// planes in the 3-D ring: with shared slopes a pass reads planes k .. k+2
+// only, unless a slip-wall zeta face on a block's upper side reads k - 1
 template <class T, int TX, int TY, bool BC>
 __host__ __device__ constexpr int stage_slots() {
   return (stage_share<T>() && !BC ? 3 : 4) + (stage_deep<T, TX, TY>() ? 1 : 0);
 }
-template <class T, int TX, int TY, bool FAST, bool VISC, bool BC>
+template <class T, int TX, int TY, bool VISC, bool BC>
 using StageSmemOf = StageSmem<T, TX, TY, (VISC && std::is_same<T, float>::value) ? 6 : 5,
                               stage_share<T>(), stage_slots<T, TX, TY, BC>()>;
 
@@ -146,7 +146,11 @@ using StageSmemOf = StageSmem<T, TX, TY, (VISC && std::is_same<T, float>::value)
 // rounds as the balanced list of the same shape.  128^3 RK step, 32 x 7 tile:
 // double-float 2.77 -> 2.46 ms, binary32 flux 0.854 -> 0.745 ms, of which the
 // block constants in shared memory (below) 6 and 9 %, as in the 32 x 8 tile.
-// (Not for the fused viscous faces, whose work hides the decoding.)
+// Not for the fused viscous faces: a sweep over tile shapes that had them by
+// rows (binary32 form with no-slip walls, 32 x 8 cells / 288 threads, 256x96x48
+// laminar O-grid) once ended in an illegal address.  Its cause was not found: no
+// bad index by reading, none in two runs of a copy that checked every global and
+// shared one.  The other kernels decode their rows with the same code.
 template <int TX, int TY, int NT>
 __host__ __device__ constexpr bool stage_rows() {
   return TX == 32 && NT == 32 * (TY + 1);
@@ -193,7 +197,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
   using MT = typename MetricStore<T>::type;
   constexpr int NV = FUSED_VISC ? 6 : 5;
   constexpr bool SHARE = stage_share<T>();
-  using SM = StageSmemOf<T, TX, TY, FAST, VISC, BC>;
+  using SM = StageSmemOf<T, TX, TY, VISC, BC>;
   constexpr int W = SM::W, PL = SM::PL;
   constexpr int NXI = SM::NXI, NETA = SM::NETA, NZETA = SM::NZETA;
   constexpr int NHX = SM::NHX, NHY = SM::NHY;
@@ -784,7 +788,7 @@ __global__ void __launch_bounds__(NT, (stage_min_ctas<T, NT, VISC>())) fv_stage_
 // creation), so a launch is a plain enqueue that stream capture accepts.
 template <class T, int TX, int TY, int NT, bool PF, bool FAST, bool VISC, bool BC, bool PLANE>
 static int launch_stage_t(const FvStageArgs& a, const FvLaunch& l, cudaStream_t s) {
-  const size_t smem = StageSmemOf<T, TX, TY, FAST, VISC, BC>::bytes(l.three_d != 0, PF);
+  const size_t smem = StageSmemOf<T, TX, TY, VISC, BC>::bytes(l.three_d != 0, PF);
   const StageC<T> c = make_stage_consts<T>(a);
   if (l.three_d) {
     if constexpr (PLANE) return -2;
@@ -797,7 +801,7 @@ static int launch_stage_t(const FvStageArgs& a, const FvLaunch& l, cudaStream_t 
 
 template <class T, int TX, int TY, int NT, bool PF, bool FAST, bool VISC, bool BC, bool PLANE>
 static int occupancy_t(bool three_d, size_t* smem_out) {
-  const size_t smem = StageSmemOf<T, TX, TY, FAST, VISC, BC>::bytes(three_d, PF);
+  const size_t smem = StageSmemOf<T, TX, TY, VISC, BC>::bytes(three_d, PF);
   int n = 0;
   if (three_d) {
     if constexpr (!PLANE) {
