@@ -361,6 +361,10 @@ int fv_autotune(fv_handle h, double dt, int reps, void* stream);
  * (0 = automatic), number of tiles, persistent CTAs}. */
 int fv_get_launch(fv_handle h, int* out4);
 
+/* The tile shape and k-chunk (fv_config's numbers) that an automatic launch
+ * stands for now; those given or autotuned otherwise.  out2 = {shape, k-chunk}. */
+int fv_get_launch_choice(fv_handle h, int* out2);
+
 /* Discrete-adjoint vector-Jacobian product of one RK stage m with step dt.
  * Stage map: Q^(m) = Q^(0) - alpha_m dt / Omega R(X(Q^(m-1))) with X the
  * ghost exchange.  Inputs: qin_dev = the stage input Q^(m-1) (packed ghosted

@@ -22,8 +22,8 @@ PRECISIONS = {"fp64": PREC_FP64, "df64": PREC_DF64, "fp32flux": PREC_FP32FLUX}
 EXPORTS = ("fv_config_default", "fv_create_blocks", "fv_destroy", "fv_last_error", "fv_state_size",
            "fv_field_size", "fv_cell_count", "fv_set_state", "fv_set_buffer", "fv_get_state", "fv_set_source",
            "fv_exchange_ghosts", "fv_residual", "fv_rk_stage", "fv_rk_step", "fv_residual_norms",
-           "fv_adjoint_vjp", "fv_autotune", "fv_get_launch", "fv_set_boundaries", "fv_set_monitor",
-           "fv_monitor_norms", "fv_stage_state", "fv_set_state_staged", "fv_graph_count",
+           "fv_adjoint_vjp", "fv_autotune", "fv_get_launch", "fv_get_launch_choice", "fv_set_boundaries",
+           "fv_set_monitor", "fv_monitor_norms", "fv_stage_state", "fv_set_state_staged", "fv_graph_count",
            "fv_probe_alu_rates", "fv_set_halo", "fv_halo_size", "fv_halo_pack", "fv_halo_unpack",
            "fv_check_rcp64", "fv_check_sqrt64", "fv_check_face_op", "fv_check_roe64", "fv_set_adjoint_arith")
 
@@ -100,6 +100,8 @@ def load_library(path: Optional[str] = None):
     L.fv_adjoint_vjp.argtypes = [vp, i32, dbl, vp, vp, vp, vp, vp]
     L.fv_autotune.argtypes = [vp, dbl, i32, vp]
     L.fv_get_launch.argtypes = [vp, ctypes.POINTER(ctypes.c_int)]
+    L.fv_get_launch_choice.argtypes = [vp, ctypes.POINTER(ctypes.c_int)]
+    L.fv_get_launch_choice.restype = i32
     L.fv_set_boundaries.argtypes = [vp, ctypes.POINTER(fv_bc_patch), i32]
     L.fv_set_monitor.argtypes = [vp, i32]
     L.fv_stage_state.argtypes = [vp, vp, vp]
@@ -129,8 +131,8 @@ def load_library(path: Optional[str] = None):
     L.fv_halo_unpack.restype = i32
     for f in ("fv_create_blocks", "fv_destroy", "fv_set_state", "fv_set_buffer", "fv_get_state", "fv_set_source",
               "fv_exchange_ghosts", "fv_residual", "fv_rk_stage", "fv_rk_step", "fv_residual_norms",
-              "fv_adjoint_vjp", "fv_autotune", "fv_get_launch", "fv_set_boundaries", "fv_set_monitor",
-              "fv_monitor_norms", "fv_stage_state", "fv_set_state_staged"):
+              "fv_adjoint_vjp", "fv_autotune", "fv_get_launch", "fv_get_launch_choice", "fv_set_boundaries",
+           "fv_set_monitor",    "fv_monitor_norms", "fv_stage_state", "fv_set_state_staged"):
         getattr(L, f).restype = i32
     _lib = L
     return L
@@ -446,6 +448,12 @@ class Solver:
         out = (ctypes.c_int * 4)()
         self._check(self._L.fv_get_launch(self._h, out))
         return {"tile": out[0], "kchunk": out[1], "tiles": out[2], "ctas": out[3]}
+
+    def launch_choice(self):
+        """(tile shape, k-chunk) that an automatic launch stands for now."""
+        out = (ctypes.c_int * 2)()
+        self._check(self._L.fv_get_launch_choice(self._h, out))
+        return out[0], out[1]
 
     def adjoint_vjp(self, stage: int, dt: float, qin, lam_out, lam_in, lam_q0, stream=None):
         self._check(self._L.fv_adjoint_vjp(self._h, int(stage), float(dt), _ptr(qin), _ptr(lam_out),

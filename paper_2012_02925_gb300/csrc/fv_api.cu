@@ -2014,6 +2014,14 @@ int fv_get_launch(fv_handle hh, int* out4) {
   return FV_OK;
 }
 
+int fv_get_launch_choice(fv_handle hh, int* out2) {
+  if (!hh || !out2) return FV_ERR_INVALID_ARG;
+  fv_ctx* h = H(hh);
+  out2[0] = h->launch.shape;
+  out2[1] = h->kchunk;
+  return FV_OK;
+}
+
 int fv_set_adjoint_arith(fv_handle hh, int precision) {
   if (!hh) return FV_ERR_INVALID_ARG;
   fv_ctx* h = H(hh);
