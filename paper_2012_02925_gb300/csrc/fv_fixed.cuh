@@ -237,13 +237,13 @@ struct FxFace {
 // Twice the flux per unit area in four numbers: the mass flux M (Q(65 + kn)),
 // the factor G of u_R - u_L (Q(65 + kn)), the dissipative pressure X (Q(67 + kn)) and
 // the energy flux E (Q(69 + kn)); the momentum flux is M u_L + G (u_R - u_L) +
-// n (p_L + p_R + X).  With the entropy fix on every eigenvalue, where |lambda_2|
-// does not get small with Vn~, they are without the waves of that eigenvalue,
-// a2 = l2 dr - t2 and a3 = l2 rt, and its parts follow: l2 (Q(64 + kl)), t2 (Q(65 + kn)),
+// n (p_L + p_R + X).  Where the entropy fix has raised |lambda_2|, which then does
+// not get small with Vn~ (fixed), they are without the waves of that eigenvalue,
+// a2 = l2 dr - t2 and a3 = l2 rt, and its parts follow: l2 (Q64), t2 (Q(65 + kn)),
 // rt (Q64) and beta (Q62).
 struct FxFlux {
   fx64 M, G, X, E, l2, t2, rt, beta;
-  int kl;
+  bool fixed;
 };
 
 // Returns nonzero when a quantity has left its range (the flux is then not to
@@ -306,9 +306,9 @@ FX_HD unsigned fx_roe(const FxConsts& C, const FxFace& f, bool fix_all, FxFlux& 
   const fx64 t2 = fx_mul(k2, P << 2);                                   // Q(58 + ls + kn)
   wild |= (fx_mag(t2) >> 1) >> (19 + ls);                               // below 1/64
   fx64 A2 = 0, a3 = 0;
-  if (fix_all) {
-    F.l2 = fixed ? fx_umul(k2 << (6 - ls), c) << 2 : (fx64)an;          // Q62 -> Q64
-    F.kl = fixed ? 0 : f.kn;
+  F.fixed = fixed;
+  if (fixed) {
+    F.l2 = fx_umul(k2 << (6 - ls), c) << 2;                             // Q62 -> Q64
     F.t2 = t2 << (7 - ls);
     F.rt = rt;
     F.beta = beta;
@@ -328,7 +328,7 @@ FX_HD unsigned fx_roe(const FxConsts& C, const FxFace& f, bool fix_all, FxFlux& 
   const fx64 hL = (HL + 2 * qL) << 2, dh = (dH + 2 * dq) << 2;          // Q68
   const fx64 G4 = mR1 - (fx_mul(beta << 1, a15) << 1);
   F.E = fx_smul(hL, M1) + fx_mul(G4, dh) - (fx_mul(d51 << 2, Vnt) >> kn);
-  if (!fix_all) {
+  if (!fixed) {
     const fx64 qt = (qL + (fx_mul(beta << 1, dq) << 1) - b2) << 3;      // q~, Q65 -> Q68
     const fx64 uw = (dq - e) + 2 * be;                                  // u~.du, Q65
     const fx64 ud = (uw << 1) - ((fx_mul(Vnt, dVn) >> kn) >> kn << 2);  // u~.du - Vn~ dVn, Q66
@@ -612,7 +612,6 @@ FX_HD bool fx_roe_flux(const FxConsts& C, const double VL[5], const double VR[5]
     f.qR += fx_usqr(b);
     f.e += fx_usqr(fx_abs(fx_sign(b, VR[i]) - fx_sign(a, VL[i])));
   }
-  fix_all = fix_all && C.eta > 0;
   FxFlux F;
   if (fx_roe(C, f, fix_all, F)) return false;
   // the area's significand, Q63 in [1/2, 1) with its top kept from rounding
@@ -626,9 +625,9 @@ FX_HD bool fx_roe_flux(const FxConsts& C, const double VL[5], const double VR[5]
   double X = fx_to_double(fx_mul(F.X, am), e - 2 + S.mv - f.kn);
   double E = fx_to_double(fx_smul(am, F.E), e - 4 + 2 * S.mv - f.kn);
   const double hA = fx_double(ah - (1 << 20), al);
-  if (fix_all) {
+  if (fix_all && F.fixed) {
     const double b = fx_to_double(F.beta, -62), dVn = VnR - VnL;
-    const double l2A = fx_to_double(F.l2, S.mv - 64 - F.kl) * hA;
+    const double l2A = fx_to_double(F.l2, S.mv - 64) * hA;
     const double a2 = fma(l2A, VR[0] - VL[0], -fx_to_double(fx_mul(F.t2, am), e - f.kn));
     const double a3 = l2A * fx_to_double(F.rt, S.mr - 64);
     double ud = -fma(b, dVn, VnL) * dVn, q = 0.0;
