@@ -12,8 +12,8 @@
 // gathers its own in a fixed order; connections are transposed one launch at
 // a time in table order.
 //
-// 96^3 VJP stage (van Albada), double-float sweeps 1.80 -> 0.87 ms, binary64
-// 4.58 -> 2.77 ms against one kernel per face that recovered its four cells'
+// 96^3 VJP stage (van Albada), double-float sweeps 1.80 -> 0.80 ms, binary64
+// 4.58 -> 2.74 ms against one kernel per face that recovered its four cells'
 // primitives, evaluated the limiter's derivatives (20 of them), and reversed
 // all of it into 20 conserved cotangents (12,700 instructions a face, 160
 // bytes written): a face now does its Roe part and writes 10 cotangents
@@ -64,7 +64,7 @@ template <> struct AdjMem<df64> {
 // the end: the high parts error-free in s, their errors and the low parts in the
 // pair (m, l).  20 binary32 operations a pair, where a binary64 addition holds
 // the FP64 unit for 80 issue slots and needs the pair converted (64 blocks of
-// 6..10 cells an axis, one VJP stage 7.37 -> 6.50 ms; 96^3 the same).  The binary64
+// 6..10 cells an axis, one VJP stage 7.37 -> 6.43 ms; 96^3 the same).  The binary64
 // parts of a cell's sum apart, in d.
 template <class T> struct AdjSum;
 template <> struct AdjSum<df64> {
@@ -202,7 +202,8 @@ __global__ void __launch_bounds__(NT, MINB) adj_face_kernel(const FvBlockDev B, 
 // component by component (the sum in binary64, the shares as the sweep's type
 // has them), one evaluation per cell, direction and variable
 // (evaluated three times, by each cell that takes a share, the 96^3 VJP stage
-// took 0.98 instead of 0.84 ms in double-float, 4.13 instead of 2.77 in binary64).
+// took 0.98 instead of 0.84 ms in double-float, 4.13 instead of 2.77 in binary64,
+// measured before the sums were binary64 again).
 template <class T>
 __global__ void __launch_bounds__(128) adj_slope_kernel(const FvBlockDev B, int dir,
                                                         const typename AdjMem<T>::type* __restrict__ prim,
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(128) adj_slope_kernel(const FvBlockDev B, int 
 // The cells' cotangents: the slope kernel's shares in a fixed order (xi, eta,
 // zeta; deterministic) and the primitive recovery's transpose, both in binary64
 // in either form (summed in double-float it would keep 48 bits, and one 96^3 VJP
-// stage with double-float sweeps take 0.76 instead of 0.87 ms).  Into lamg for
+// stage with double-float sweeps take 0.76 instead of 0.80 ms).  Into lamg for
 // every ghosted cell; or, when no connection has to be transposed (lam_in not
 // null), straight to lam_in for the interior cells, with lam_q0 += lam_out.
 template <class T>
@@ -271,6 +272,7 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const
   const bool ii = i >= 0 && i < B.ni, jj = j >= 0 && j < B.nj, kk = k >= 0 && k < B.nk;
   const long long gx = B.qoff + ghost_index(B, i, j, k);
   AdjSum<T> share[5];
+  const T zero = Sc<T>::c(0.0);
 #pragma unroll 1
   for (int dir = 0; dir < 2 + three_d; ++dir) {
     if (!(dir == 0 ? jj && kk : (dir == 1 ? ii && kk : ii && jj))) continue;
@@ -281,11 +283,21 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const FvBlockDev B, const
     const long long nc = ci * cj * ck, st = dir == 0 ? 1 : (dir == 1 ? ci : ci * cj);
     const long long c = ((long long)(k + (dir == 2)) * cj + (j + (dir == 1))) * ci + (i + (dir == 0));
     const bool at = p >= -1 && p <= nd, lo = p >= 0 && p <= nd + 1, up = p >= -2 && p <= nd - 1;
+    // all fifteen loads of the direction in flight before the first sum (loaded
+    // where each is added, one after the other: 96^3 VJP stage 0.87 instead of 0.80 ms)
+    double o[5];
+    T a[5], b[5];
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
-      if (at) share[q].add(__ldg(own + q * nc + c));
-      if (lo) share[q].add(M::ld(s + (5 + q) * nc + c - st));
-      if (up) share[q].sub(M::ld(s + (10 + q) * nc + c + st));
+      o[q] = at ? __ldg(own + q * nc + c) : 0.0;
+      a[q] = lo ? M::ld(s + (5 + q) * nc + c - st) : zero;
+      b[q] = up ? M::ld(s + (10 + q) * nc + c + st) : zero;
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      share[q].add(o[q]);
+      share[q].add(a[q]);
+      share[q].sub(b[q]);
     }
   }
   double Vb[5];
