@@ -914,15 +914,17 @@ int kchunk_of(const FvBlockDev& b, int dim, int kchunk, long long slots, long lo
 // latencies: with `ref` resident CTAs (those of the measurement) or fewer a
 // tile-plane takes ref x cost x cells, and a wave of tiles the same whether
 // or not every slot has one; many more tiles than slots even out (dynamic
-// hand-out), up to half a tile at the end.  Costs per cell and plane:
+// hand-out), up to half a tile at the end.  Costs per cell and plane: ratios of
 // measured RK steps of the 128^3 block and (2-D) of the 1100 x 300 inlet,
-// which fill the chip in every shape.  Measured on 15 problems from 1,024 to
-// 10.9 M cells, RK step with the fixed 32 x 8 shape (16 x 8 for narrow blocks)
-// over this rule's: binary64 1.2 .. 2.5, double-float 1.0 .. 2.2,
-// binary32 flux 1.0 .. 2.0; 64-block batch in binary64 39.3 -> 24.7 ms, in
-// binary32 flux 5.23 -> 4.74 ms.  (8 x 8 with 160 threads, 2-D: its cost makes
-// it the choice while every tile has a slot at once; 64^2 vortex 70 -> 58 us,
-// at 192^2 it would take 105 us where the rule's pick takes 93.)
+// which fill the chip in every shape, except shape 13's (8 x 8 with 160 threads,
+// 2-D) and binary32 flux's two corrections below: those are fitted so that the
+// choice flips where the times do (shape 13 while every tile has a slot at once:
+// 64^2 vortex 70 -> 58 us; at 192^2 it would take 105 us where the rule's pick
+// takes 93).  RK step with the fixed 32 x 8 shape (16 x 8 for narrow blocks) over
+// this rule's, 15 problems from 1,024 to 10.9 M cells: binary64 1.2 .. 2.5,
+// double-float 1.0 .. 2.2, binary32 flux 1.0 .. 2.0.  Over the fastest of the
+// compiled shapes and k-chunks, 13 problems in three forms: within 1.3 % in 33
+// of 39, within 5.4 % in 38; a 48^3 block in double-float takes 11 % longer.
 void choose_launch(fv_ctx* h) {
   const fv_config& c = h->cfg;
   FvLaunch l{};
