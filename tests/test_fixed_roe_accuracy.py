@@ -177,7 +177,7 @@ def test_entropy_fix_on_every_eigenvalue(fluxes, mach, jump, harten):
 
 @pytest.mark.parametrize("fix_all", [0, 1])
 @pytest.mark.parametrize("mach", [0.01, 0.1, 1.0, 3.0])
-@pytest.mark.parametrize("kind", ["strong", "contact", "shear"])
+@pytest.mark.parametrize("kind", ["strong", "contact", "shear", "opposed"])
 def test_large_jumps(fluxes, kind, mach, fix_all):
     rng = np.random.default_rng(6)
     x = faces(rng, N, mach, 0.5, 0.5, axis=kind == "shear")
@@ -187,6 +187,9 @@ def test_large_jumps(fluxes, kind, mach, fix_all):
         x[:, 9] = x[:, 4]
     if kind == "contact":
         x[:, 6:9] = x[:, 1:4]
+    if kind == "opposed":      # the averaged velocity is zero up to rounding
+        x[:, 5] = x[:, 0] * (1 + 1e-9 * rng.uniform(-1, 1, N))
+        x[:, 6:9] = -x[:, 1:4]
     if kind == "shear":
         x[:, 5] = x[:, 0]
         k = np.abs(x[:, 10:13]).argmax(axis=1)
@@ -247,3 +250,38 @@ def test_reflections(fluxes, mach):
     a, b = fluxes(x)[1], fluxes(y)[1]
     for i in (0, 4):
         assert (np.abs(a[:, i] + b[:, i]) <= np.spacing(np.abs(a[:, i]))).all()
+
+
+def test_any_face_it_takes(fluxes):
+    """Faces of all kinds - jumps of 1e-16 to ten times, equal or opposed states,
+    components 1e-200 of the others: what the fixed point takes is right to 16 units of
+    2^-53 of the flux's scale rho (|u| + c)^a."""
+    rng = np.random.default_rng(9)
+    n = 200000
+    for gamma, harten, fix_all in ((1.3, 0.95, 1), (1.4, 0.1, 0), (5.0 / 3.0, 0.0, 1), (1.95, 0.0626, 1)):
+        mach = 10.0 ** rng.uniform(-8, 1.2, (n, 1))
+        x = faces(rng, n, 1.0, 0.0, gamma=gamma)
+        x[:, 1:4] *= mach
+        tiny = rng.random((n, 3)) < 0.1
+        x[:, 1:4] *= np.where(tiny, 10.0 ** rng.uniform(-200, 0, (n, 3)), 1.0)
+        axis = rng.random(n) < 0.3
+        x[axis, 10:13] = np.eye(3)[rng.integers(0, 3, axis.sum())]
+        speed = np.linalg.norm(x[:, 1:4], axis=1, keepdims=True)
+        j = 10.0 ** rng.uniform(-16, 0, (n, 1))
+        x[:, 5:6] = x[:, 0:1] * np.exp(j * rng.uniform(-1, 1, (n, 1)))
+        x[:, 6:9] = x[:, 1:4] + j * speed * rng.uniform(-1, 1, (n, 3))
+        x[:, 9:10] = x[:, 4:5] * np.exp(np.where(rng.random((n, 1)) < 0.3, 10.0, 1.0) * j * rng.uniform(-1, 1, (n, 1)))
+        kind = rng.integers(0, 6, n)
+        x[kind == 0, 9] = x[kind == 0, 4]
+        x[kind == 1, 5] = x[kind == 1, 0]
+        x[kind == 2, 6:9] = x[kind == 2, 1:4]
+        x[kind == 3, 6:9] = -x[kind == 3, 1:4]
+        taken, flux, ef, eb = fluxes(x, gamma, harten, fix_all)
+        assert taken > 0.8 * n
+        # errors are in units of rho_L c_L^a; the flux's scale has both sides and the speed
+        c = np.sqrt(gamma * x[:, [4, 9]] / x[:, [0, 5]])
+        u = np.stack([np.linalg.norm(x[:, 1:4], axis=1), np.linalg.norm(x[:, 6:9], axis=1)], axis=1)
+        S = (u.max(axis=1) + c.max(axis=1)) / c[:, 0]
+        scale = (np.maximum(x[:, 0], x[:, 5]) / x[:, 0])[:, None] * np.stack([S, S ** 2, S ** 2, S ** 2, S ** 3], axis=1)
+        on = np.isfinite(flux[:, 0])
+        assert np.nanmax(np.abs(ef[on]) / scale[on]) <= 16 * 2.0 ** -53
